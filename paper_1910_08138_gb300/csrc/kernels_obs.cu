@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "rpba_internal.cuh"
 
 namespace rpba {
@@ -560,177 +562,294 @@ __device__ __noinline__ bool point_normal_fp64(const View &v, int j, double *N, 
   return ok;
 }
 
-// per instance of a running point: partial normal matrix N^(l) (sym3) and
-// gradient g^(l) at the current X_j, cameras fixed. flag bit: behind camera.
-template <typename T>
-__global__ void k_isect_inst(View v, const int *state, T *part) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= v.P) return;
-  int j = v.inst_pt[q];
-  if (state[j] != 1) return;
-  T N[6] = {0, 0, 0, 0, 0, 0}, g[3] = {0, 0, 0};
-  bool behind = false;
-  for (int k = v.inst_obs_ptr[q]; k < v.inst_obs_ptr[q + 1]; k++) {
-    int i = v.obs_cam[k];
-    ProjX<T> pj;
-    T z;
-    proj_x<T>(v, i, v.X + 3 * j, v.X_hi + 3 * j, v.X_lo + 3 * j, pj, z);
-    if (!(z > T(0))) { behind = true; continue; }
-    ObsT<T> ob;
-    load_obs<T>(v, k, ob);
-    T r0 = pj.u - ob.x, r1 = pj.v - ob.y;
-    // w W Jx (2x3)
-    T a0[3], a1[3];
-    for (int c = 0; c < 3; c++) {
-      a0[c] = ob.w * (ob.W[0] * pj.Jx[c] + ob.W[1] * pj.Jx[3 + c]);
-      a1[c] = ob.w * (ob.W[1] * pj.Jx[c] + ob.W[2] * pj.Jx[3 + c]);
-    }
-    for (int r = 0; r < 3; r++) {
-      for (int c = r; c < 3; c++) N[s3idx(r, c)] += pj.Jx[r] * a0[c] + pj.Jx[3 + r] * a1[c];
-      g[r] += a0[r] * r0 + a1[r] * r1;
-    }
-  }
-  T *o = part + 10 * (size_t)q;
-  for (int e = 0; e < 6; e++) o[e] = N[e];
-  for (int e = 0; e < 3; e++) o[6 + e] = g[e];
-  o[9] = behind ? T(-1) : T(v.inst_obs_ptr[q + 1] - v.inst_obs_ptr[q]);  // observation count
+// FP64 form and every form's first intersection: the Gauss-Newton iterations
+// of Eq. bars, cameras fixed, all in one launch. FP64 instructions bound it
+// (1/64 of the FP32 rate on this GPU, compares included, and a warp's
+// instruction holds the pipe for 16 cycles however few of its lanes are
+// active), so the layout keeps lanes full and the instructions few:
+//   - a CTA takes a tile of up to ISECT_D_TILE points; per iteration the
+//     observations of the points still running are flattened over its threads,
+//     one each, whatever the track lengths. Most points converge in two or
+//     three iterations and a few outlier points take ten: with one thread per
+//     point nearly every warp waited for such a point.
+//   - the observations' terms of N_j and g_j go through shared memory, and
+//     each of the nine sums of a point is added up by one thread in the
+//     order of the observations and instances (the sums do not depend on the
+//     tile or the chunks);
+//   - one thread per running point solves, checks and updates.
+//   - products that cannot change a value are left out (C^-1 = I without
+//     observation weights, w = 1), tests of a sign or of w are taken on the
+//     bits, and square roots only where exponents do not already decide.
+// The first intersection, before (two kernels over all instances and points
+// per iteration) -> now: 10,000 cameras with 2.0M observations 5.51 -> 1.34 ms,
+// 1,000 cameras with 600k 1.38 -> 0.37 ms, 961 cameras with per-camera
+// intrinsics and tracks of 18 (360k) 1.65 -> 0.41 ms, 50 cameras 0.36 -> 0.08 ms.
+// One thread per point with shrinking lists of running points took 3.0 ms on
+// the first and 3 ms on the third of these.
+#define ISECT_D_THREADS 128
+#define ISECT_D_TILE 128
+
+__device__ __forceinline__ bool d_positive(double x) {
+  long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
-// per running point: sum the instance parts, Gauss-Newton update, checks,
-// and on convergence W^l = N - N^(l) for every instance. Converged when
-// ||dX|| <= tol (1 + ||X||) or when the step moves the point's image
-// residuals by less than px_tol per observation: dX^T N dX <= px_tol^2 n_obs
-// (reachable in FP32, whose residuals carry ~1e-4 px rounding).
-// FP32 form: the 3x3 system is solved in FP32; when its Frobenius condition
-// number exceeds 1e6, N_j and g_j are formed again in FP64 from the
-// observations, and the cond_max test and the solve use those.
-template <typename T>
-__global__ void k_isect_point(View v, int *state, int *iter, const T *part, int max_iter, double tol,
-                              double px_tol, double cond_max, int last) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= v.N || state[j] != 1) return;
-  int q0 = v.pt_inst_ptr[j], q1 = v.pt_inst_ptr[j + 1];
-  T N[6] = {0, 0, 0, 0, 0, 0}, g[3] = {0, 0, 0};
-  bool behind = false;
-  T nobs = 0;
-  for (int a = q0; a < q1; a++) {
-    const T *o = part + 10 * (size_t)v.pt_inst[a];
-    for (int e = 0; e < 6; e++) N[e] += o[e];
-    for (int e = 0; e < 3; e++) g[e] += o[6 + e];
-    behind |= o[9] < T(0);
-    nobs += o[9];
-  }
-  bool fail = behind;
-  double d[3] = {0, 0, 0};
-  float df[3] = {0.f, 0.f, 0.f};  // FP32 form: the step in FP32
-  double nd2_img = 0.0;           // d^T N d (FP64 re-formation)
-  T nd2T = T(-1);                 // d^T N d in the compute precision (else)
-  if (!fail) {
-    T inv[6];
-    T det = sym3_inv<T>(N, inv);
-    T cond = sym3_frob<T>(N) * sym3_frob<T>(inv);
-    double Nimg[6];
-    if (sizeof(T) == sizeof(float) && !(cond <= T(1e6))) {
-      // FP32 sums round a nearly singular N_j into a better conditioned one,
-      // so the cond_max test cannot be taken on them: N_j and g_j again in FP64
-      double gd[3], invd[6];
-      fail = !point_normal_fp64(v, j, Nimg, gd);
-      double detd = sym3_inv<double>(Nimg, invd);
-      fail = fail || !(detd > 0.0) || !(sym3_frob<double>(Nimg) * sym3_frob<double>(invd) <= cond_max);
-      for (int r = 0; r < 3; r++) {
-        d[r] = invd[s3idx(r, 0)] * gd[0] + invd[s3idx(r, 1)] * gd[1] + invd[s3idx(r, 2)] * gd[2];
-        df[r] = (float)d[r];
-      }
-      if (px_tol > 0.0) {
-        double Nd3[3];
-        for (int r = 0; r < 3; r++) Nd3[r] = Nimg[s3idx(r, 0)] * d[0] + Nimg[s3idx(r, 1)] * d[1] + Nimg[s3idx(r, 2)] * d[2];
-        nd2_img = d[0] * Nd3[0] + d[1] * Nd3[1] + d[2] * Nd3[2];
-      }
-    } else {
-      // the step and its image-space size in the compute precision; only the
-      // position update below is FP64
-      fail = !(det > T(0)) || !(cond <= (T)cond_max);
-      T dT[3];
-      for (int r = 0; r < 3; r++) dT[r] = inv[s3idx(r, 0)] * g[0] + inv[s3idx(r, 1)] * g[1] + inv[s3idx(r, 2)] * g[2];
-      if (px_tol > 0.0) {
-        T Nd3[3];
-        for (int r = 0; r < 3; r++) Nd3[r] = N[s3idx(r, 0)] * dT[0] + N[s3idx(r, 1)] * dT[1] + N[s3idx(r, 2)] * dT[2];
-        nd2T = dT[0] * Nd3[0] + dT[1] * Nd3[1] + dT[2] * Nd3[2];
-      }
-      if constexpr (sizeof(T) == sizeof(float))
-        for (int r = 0; r < 3; r++) df[r] = (float)dT[r];
-      else
-        for (int r = 0; r < 3; r++) d[r] = (double)dT[r];
+// the terms of observation k in N (6, upper) and g (3) at X; false when it
+// lies behind its camera
+template <bool WINV, int CD>
+__device__ __forceinline__ bool isect_terms_d(const View &v, const double X[3], int k, double (&o)[9]) {
+  int i = v.obs_cam[k];
+  ProjJac<double, CD> pj;
+  double z;
+  obs_proj<double, CD>(v, i, X, nullptr, nullptr, pj, z);
+  double r0 = pj.u - (v.obs_xy[2 * (size_t)k] - v.intr[3 * i + 1]);
+  double r1 = pj.v - (v.obs_xy[2 * (size_t)k + 1] - v.intr[3 * i + 2]);
+  double a0[3], a1[3];  // w W Jx (2x3)
+  if constexpr (WINV) {
+    const double *W = v.obs_winv + 3 * (size_t)k;
+    double W0 = W[0], W1 = W[1], W2 = W[2];
+    for (int c = 0; c < 3; c++) {
+      a0[c] = W0 * pj.Jx[c] + W1 * pj.Jx[3 + c];
+      a1[c] = W1 * pj.Jx[c] + W2 * pj.Jx[3 + c];
     }
+  } else {
+    for (int c = 0; c < 3; c++) { a0[c] = pj.Jx[c]; a1[c] = pj.Jx[3 + c]; }
   }
+  double w = v.obs_w[k];
+  if (__double_as_longlong(w) != 0x3ff0000000000000ll)  // w != 1
+    for (int c = 0; c < 3; c++) { a0[c] = w * a0[c]; a1[c] = w * a1[c]; }
+  for (int r = 0; r < 3; r++) {
+    for (int c = r; c < 3; c++) o[s3idx(r, c)] = pj.Jx[r] * a0[c] + pj.Jx[3 + r] * a1[c];
+    o[6 + r] = a0[r] * r0 + a1[r] * r1;
+  }
+  return d_positive(z);
+}
+
+// biased exponent of the largest magnitude of n values (2047 for inf or NaN):
+// max |x| < 2^(e - 1022), and max |x| >= 2^(e - 1023) for e > 0
+template <int NV>
+__device__ __forceinline__ int max_exponent(const double (&x)[NV]) {
+  int e = 0;
+#pragma unroll
+  for (int k = 0; k < NV; k++) e = max(e, (__double2hiint(x[k]) >> 20) & 0x7ff);
+  return e;
+}
+
+// The 3x3 solve of one point, its checks and its update. Converged when
+// ||dX|| <= tol (1 + ||X||) or when the step moves the point's image residuals
+// by less than px_tol per observation: dX^T N dX <= px_tol^2 n_obs. Returns
+// the point's state: 1 running, 2 converged, 3 failed.
+__device__ __forceinline__ int isect_solve_d(const double (&N)[6], const double (&g)[3], double (&X)[3], bool &moved,
+                                             int nobs, double tol, double px_tol, double cond_max, int cond_exp,
+                                             bool last) {
+  double inv[6], d[3];
+  double det = sym3_inv<double>(N, inv);
+  // ||N||_F ||N^-1||_F <= 9 max|N| max|N^-1| < 2^(eN + eI - 2040)
+  bool ok = d_positive(det);
+  int eN = max_exponent(N), eI = max_exponent(inv);
+  if (ok && (eN + eI - 2040 > cond_exp || max(eN, eI) == 2047))
+    ok = sym3_frob<double>(N) * sym3_frob<double>(inv) <= cond_max;
+  if (!ok) return 3;
+  for (int r = 0; r < 3; r++) d[r] = inv[s3idx(r, 0)] * g[0] + inv[s3idx(r, 1)] * g[1] + inv[s3idx(r, 2)] * g[2];
+  for (int r = 0; r < 3; r++) X[r] = X[r] - d[r];
+  moved = true;
   bool conv = false;
-  if (!fail) {
-    if constexpr (sizeof(T) == sizeof(float)) {
-      // X - d on the hi + lo words in float-float; the FP64 copy from them
-      float *xh = v.X_hi + 3 * j, *xl = v.X_lo + 3 * j;
-      for (int r = 0; r < 3; r++) {
-        float2 xn = ff_add(make_float2(xh[r], xl[r]), make_float2(-df[r], 0.f));
-        xh[r] = xn.x;
-        xl[r] = xn.y;
-        v.X[3 * j + r] = ff_to_double(xn);
-      }
-      float nd = sqrtf(df[0] * df[0] + df[1] * df[1] + df[2] * df[2]);
-      float nx = sqrtf(xh[0] * xh[0] + xh[1] * xh[1] + xh[2] * xh[2]);
-      conv = nd <= (float)tol * (1.f + nx);
-    } else {
-      double Xn[3];
-      for (int r = 0; r < 3; r++) Xn[r] = v.X[3 * j + r] - d[r];
-      for (int r = 0; r < 3; r++) v.X[3 * j + r] = Xn[r];
-      if (v.X_hi)  // FP32 form under its FP64 first intersection: the hi + lo mirror
-        for (int r = 0; r < 3; r++) split(Xn[r], v.X_hi[3 * j + r], v.X_lo[3 * j + r]);
+  if (px_tol > 0.0) {
+    double Nd3[3];
+    for (int r = 0; r < 3; r++) Nd3[r] = N[s3idx(r, 0)] * d[0] + N[s3idx(r, 1)] * d[1] + N[s3idx(r, 2)] * d[2];
+    double nd2 = d[0] * Nd3[0] + d[1] * Nd3[1] + d[2] * Nd3[2];
+    conv = (nd2 >= 0.0 ? nd2 : 0.0) <= px_tol * px_tol * (double)nobs;
+  }
+  // ||dX|| >= 2^(ed - 1023), tol < 2^(et - 1022), 1 + ||X|| < 2^(ex - 1020)
+  if (!conv) {
+    int ed = max_exponent(d), ex = max(max_exponent(X), 1023), et = (__double2hiint(tol) >> 20) & 0x7ff;
+    if (ed - 1023 < (et - 1022) + (ex - 1020) || ed == 2047) {
       double nd = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      double nx = sqrt(Xn[0] * Xn[0] + Xn[1] * Xn[1] + Xn[2] * Xn[2]);
+      double nx = sqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
       conv = nd <= tol * (1.0 + nx);
     }
-    if (!conv && px_tol > 0.0)
-      conv = nd2T >= T(0) ? nd2T <= (T)(px_tol * px_tol) * nobs : nd2_img <= px_tol * px_tol * (double)nobs;
   }
-  int it = ++iter[j];
-  if (!fail && !conv && (it >= max_iter || last)) fail = true;
-  if (fail) {
-    state[j] = 3;
-    v.active[j] = 0;
-    for (int a = q0; a < q1; a++)
-      for (int e = 0; e < 6; e++) {
-        v.Wl[6 * (size_t)v.pt_inst[a] + e] = 0.0;
-        if (v.Wl32) v.Wl32[6 * (size_t)v.pt_inst[a] + e] = 0.f;
+  return conv ? 2 : last ? 3 : 1;
+}
+
+template <bool WINV, int CD>
+__global__ void __launch_bounds__(ISECT_D_THREADS)
+    k_isect_fused_d(View v, const int *list, int n, int tile, const int *pt_obs_ptr, const int *pt_obs,
+                    const uint8_t *pt_mask, int *state, int *iter, int max_iter, double tol, double px_tol,
+                    double cond_max, int cond_exp) {
+  __shared__ double term[9][ISECT_D_THREADS];                         // of the chunk's observations
+  __shared__ double part[9][ISECT_D_TILE], total[9][ISECT_D_TILE];    // per running point: instance, point
+  __shared__ double xs[3][ISECT_D_TILE];
+  __shared__ int end_inst[ISECT_D_THREADS];                           // instance that ends here, or -1
+  __shared__ int pj[ISECT_D_TILE], pre[ISECT_D_TILE + 1], behind[ISECT_D_TILE], wsum[ISECT_D_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int t0 = blockIdx.x * tile, nt = min(tile, n - t0);
+  // the running points, compacted in order: thread tid holds (j, X) of slot tid
+  // after every compaction
+  int j = -1;
+  bool run = false, moved = false;
+  double X[3] = {0, 0, 0};
+  if (tid < nt) {
+    j = list ? list[t0 + tid] : t0 + tid;
+    if (pt_mask) {
+      run = v.active[j] && pt_mask[j];
+      iter[j] = 0;
+      if (!run || max_iter <= 0) state[j] = run ? 1 : 0;
+    } else {
+      run = state[j] == 1;
+    }
+    for (int e = 0; e < 3; e++) X[e] = v.X[3 * (size_t)j + e];
+  }
+  for (int it = 1; it <= max_iter; it++) {
+    // compaction of the running points and the prefix sums of their observations
+    unsigned left = __ballot_sync(0xffffffffu, run);
+    if (lane == 0) wsum[wid] = __popc(left);
+    __syncthreads();
+    int nrun = 0, slot = __popc(left & ((1u << lane) - 1u));
+#pragma unroll
+    for (int w = 0; w < ISECT_D_THREADS / 32; w++) {
+      if (w < wid) slot += wsum[w];
+      nrun += wsum[w];
+    }
+    if (nrun == 0) return;
+    if (run) {
+      pj[slot] = j;
+      for (int e = 0; e < 3; e++) xs[e][slot] = X[e];
+    }
+    __syncthreads();
+    int cnt = 0;
+    if (tid < nrun) {
+      j = pj[tid];
+      for (int e = 0; e < 3; e++) X[e] = xs[e][tid];
+      cnt = pt_obs_ptr[j + 1] - pt_obs_ptr[j];
+      behind[tid] = 0;
+    }
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[wid] = incl;
+    for (int e = tid; e < 9 * ISECT_D_TILE; e += ISECT_D_THREADS) {
+      (&part[0][0])[e] = 0.0;
+      (&total[0][0])[e] = 0.0;
+    }
+    __syncthreads();
+    int base = 0;
+#pragma unroll
+    for (int w = 0; w < ISECT_D_THREADS / 32; w++)
+      if (w < wid) base += wsum[w];
+    if (tid < nrun) pre[tid + 1] = base + incl;
+    if (tid == 0) pre[0] = 0;
+    __syncthreads();
+    const int nobs = pre[nrun];
+    for (int c0 = 0; c0 < nobs; c0 += ISECT_D_THREADS) {
+      const int o = c0 + tid, c1 = min(c0 + ISECT_D_THREADS, nobs);
+      if (o < nobs) {
+        int lo = 0, hi = nrun - 1;  // the slot with pre[slot] <= o < pre[slot + 1]
+        while (lo < hi) {
+          int mid = (lo + hi + 1) >> 1;
+          if (pre[mid] <= o) lo = mid; else hi = mid - 1;
+        }
+        unsigned code = (unsigned)pt_obs[pt_obs_ptr[pj[lo]] + (o - pre[lo])];
+        int k = (int)(code & 0x7fffffffu);
+        double Xo[3] = {xs[0][lo], xs[1][lo], xs[2][lo]}, tm[9];
+        if (!isect_terms_d<WINV, CD>(v, Xo, k, tm)) behind[lo] = 1;
+#pragma unroll
+        for (int e = 0; e < 9; e++) term[e][tid] = tm[e];
+        end_inst[tid] = (code & 0x80000000u) ? v.obs_inst[k] : -1;
       }
-  } else if (conv) {
-    state[j] = 2;
-    bool tp = (q1 - q0) >= 2;
-    for (int a = q0; a < q1; a++) {
-      int q = v.pt_inst[a];
-      const T *o = part + 10 * (size_t)q;
-      if constexpr (sizeof(T) == sizeof(float)) {
-        // FP32 form: W^l as the float-float sum of the other instances' parts.
-        // N - N^(l) in FP32 cancels when the other sub-blocks' observations are
-        // down-weighted (w = 1e-4), and can lose positive semi-definiteness.
-        float Wh[6] = {0, 0, 0, 0, 0, 0}, Wlo[6] = {0, 0, 0, 0, 0, 0};
-        for (int b = q0; b < q1; b++) {
-          if (b == a) continue;
-          const T *ob = part + 10 * (size_t)v.pt_inst[b];
-          for (int e = 0; e < 6; e++) ff_acc(Wh[e], Wlo[e], ob[e]);
+      __syncthreads();
+      // the chunk's points: [s0, s1), nine sums each
+      int s0, s1;
+      {
+        int lo = 0, hi = nrun - 1;
+        while (lo < hi) {
+          int mid = (lo + hi + 1) >> 1;
+          if (pre[mid] <= c0) lo = mid; else hi = mid - 1;
         }
-        for (int e = 0; e < 6; e++) {
-          float2 w = make_float2(Wh[e], Wlo[e]);
-          double wd = tp_weight(v, e, ff_to_double(w), (double)N[e]);
-          v.Wl[6 * (size_t)q + e] = tp ? wd : 0.0;
-          v.Wl32[6 * (size_t)q + e] = tp ? (v.wmode ? (float)wd : __fadd_rn(Wh[e], Wlo[e])) : 0.f;
+        s0 = lo;
+        lo = s0;
+        hi = nrun - 1;
+        while (lo < hi) {
+          int mid = (lo + hi + 1) >> 1;
+          if (pre[mid] <= c1 - 1) lo = mid; else hi = mid - 1;
         }
-      } else {
-        for (int e = 0; e < 6; e++)
-          v.Wl[6 * (size_t)q + e] = tp ? tp_weight(v, e, (double)(N[e] - o[e]), (double)N[e]) : 0.0;
-        if (v.Wl32)
-          for (int e = 0; e < 6; e++)
-            v.Wl32[6 * (size_t)q + e] = tp ? (float)tp_weight(v, e, (double)(N[e] - o[e]), (double)N[e]) : 0.f;
+        s1 = lo + 1;
+      }
+      const int ns = s1 - s0;
+      for (int e = tid; e < 9 * ns; e += ISECT_D_THREADS) {
+        int c = e / ns, sl = s0 + (e - c * ns);
+        double p = part[c][sl];
+        for (int q = max(pre[sl], c0); q < min(pre[sl + 1], c1); q++) {
+          p += term[c][q - c0];
+          int inst = end_inst[q - c0];
+          if (inst >= 0) {
+            total[c][sl] += p;
+            // the instance's part waits in its W^l slot for the refined weight
+            // (every point ends converged or failed, which overwrites it)
+            if (c < 6) v.Wl[6 * (size_t)inst + c] = p;
+            p = 0.0;
+          }
+        }
+        part[c][sl] = p;
+      }
+      __syncthreads();
+    }
+    run = false;
+    if (tid < nrun) {
+      double N[6], g[3];
+      for (int e = 0; e < 6; e++) N[e] = total[e][tid];
+      for (int e = 0; e < 3; e++) g[e] = total[6 + e][tid];
+      moved = it > 1;
+      int st = (behind[tid] || cnt == 0) ? 3
+                                         : isect_solve_d(N, g, X, moved, cnt, tol, px_tol, cond_max, cond_exp,
+                                                         it == max_iter);
+      run = st == 1;
+      if (!run) {
+        state[j] = st;
+        iter[j] = it;
+        if (moved)
+          for (int e = 0; e < 3; e++) {
+            v.X[3 * (size_t)j + e] = X[e];
+            if (v.X_hi) split(X[e], v.X_hi[3 * (size_t)j + e], v.X_lo[3 * (size_t)j + e]);
+          }
+        // W^l = N - N^(l) for every instance of a tie point, zero otherwise
+        if (st == 3) v.active[j] = 0;
+        int q0 = v.pt_inst_ptr[j], q1 = v.pt_inst_ptr[j + 1];
+        const bool tp = st == 2 && q1 - q0 >= 2;
+        for (int a = q0; a < q1; a++) {
+          double *W = v.Wl + 6 * (size_t)v.pt_inst[a];
+          for (int e = 0; e < 6; e++) {
+            double wd = tp ? tp_weight(v, e, N[e] - W[e], N[e]) : 0.0;
+            W[e] = wd;
+            if (v.Wl32) v.Wl32[6 * (size_t)v.pt_inst[a] + e] = (float)wd;
+          }
+        }
       }
     }
   }
+}
+
+// the observations by point (CSR over the internal point numbers), a point's
+// instances in order; the top bit marks the last observation of an instance
+__global__ void k_point_obs(View v, const int *ptr, int *out) {
+  int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= v.N) return;
+  int at = ptr[j];
+  for (int a = v.pt_inst_ptr[j]; a < v.pt_inst_ptr[j + 1]; a++) {
+    int q = v.pt_inst[a];
+    for (int k = v.inst_obs_ptr[q]; k < v.inst_obs_ptr[q + 1]; k++)
+      out[at++] = k + 1 < v.inst_obs_ptr[q + 1] ? k : (int)((unsigned)k | 0x80000000u);
+  }
+}
+
+rpba_status point_obs_setup(Ctx *ctx) {
+  if (ctx->N)
+    RPBA_KERNEL(ctx, "k_point_obs", k_point_obs<<<(ctx->N + 255) / 256, 256, 0, ctx->stream>>>(
+                                        make_view(ctx), ctx->pt_obs_ptr, ctx->pt_obs));
+  return RPBA_OK;
 }
 
 // FP32 form, one Gauss-Newton iteration of Eq. bars for one point (the
@@ -908,37 +1027,48 @@ __global__ void k_isect_count(const int *state, int n, int *running, int *failed
   if (state[j] == 3) atomicAdd(failed, 1);
 }
 
+// The tile: as many points per CTA as leave four CTAs for each of the 152 SMs
+// (their barriers overlap, and a small block spreads over the chip), up to
+// ISECT_D_TILE.
+template <bool WINV, int CD>
+static rpba_status isect_fp64(Ctx *ctx, const View &v, const int *list, int n, const uint8_t *pt_mask) {
+  const double cond_max = ctx->opt.cond_max;
+  // cond_max >= 2^cond_exp (below every exponent when it is not a positive number)
+  int cond_exp = cond_max > 0.0 && isfinite(cond_max) ? ilogb(cond_max) : -100000;
+  int tile = std::min(ISECT_D_TILE, std::max(16, n / (4 * 152) / 16 * 16));
+  RPBA_KERNEL(ctx, "k_isect_fused_d", (k_isect_fused_d<WINV, CD><<<nblk(n, tile), ISECT_D_THREADS, 0, ctx->stream>>>(
+                                         v, list, n, tile, ctx->pt_obs_ptr, ctx->pt_obs, pt_mask, ctx->isect_state,
+                                         ctx->isect_iter, ctx->opt.isect_max_iter, ctx->opt.isect_tol,
+                                         ctx->opt.isect_px_tol, cond_max, cond_exp)));
+  return RPBA_OK;
+}
+
 rpba_status launch_intersect(Ctx *ctx, int tp_only, int *n_dropped, bool fp64, bool tp_copies) {
   View v = make_view(ctx);
   if (ctx->N == 0) { if (n_dropped) *n_dropped = 0; return RPBA_OK; }
   const bool fused = ctx->opt.precision == 1 && !fp64;
-  // the TP list launch sets its points' start states itself unless the
-  // dropped points are counted afterwards (that count reads every state)
-  const bool own_start = fused && tp_only && !n_dropped;
+  const int *list = tp_only ? ctx->tp_list : nullptr;
+  int n = tp_only ? ctx->n_tp : ctx->N;
+  // the launches set their points' start states themselves unless the dropped
+  // points of a TP list are counted afterwards (that count reads every state)
+  const bool own_start = fused ? tp_only && !n_dropped : !(tp_only && n_dropped);
   if (!own_start) {
     RPBA_CUDA(cudaMemsetAsync(ctx->counters, 0, 4 * sizeof(int), ctx->stream));
     RPBA_KERNEL(ctx, "k_isect_start", k_isect_start<<<nblk(ctx->N, 256), 256, 0, ctx->stream>>>(
                                           v, ctx->pt_mask, ctx->isect_state, ctx->isect_iter, tp_only, ctx->counters));
   }
-  int maxit = ctx->opt.isect_max_iter;
-  double tol = ctx->opt.isect_tol;
-  double px_tol = ctx->opt.isect_px_tol;
+  const uint8_t *mask = own_start ? ctx->pt_mask : nullptr;
   if (fused) {  // FP32 form: every point's iterations in one launch
-    const int *list = tp_only ? ctx->tp_list : nullptr;
-    int n = tp_only ? ctx->n_tp : ctx->N;
     if (n)
       RPBA_KERNEL(ctx, "k_isect_fused_f", k_isect_fused_f<<<nblk(n, ctx->tune.isect), ctx->tune.isect, 0, ctx->stream>>>(
-                                            v, list, n, own_start ? ctx->pt_mask : nullptr, tp_copies && tp_only ? 1 : 0,
-                                            ctx->isect_state, ctx->isect_iter, maxit, tol, px_tol,
-                                            ctx->opt.cond_max));
-  } else {
-    for (int it = 0; it < maxit; it++) {
-      RPBA_KERNEL(ctx, "k_isect_inst", k_isect_inst<double><<<nblk(ctx->P, 128), 128, 0, ctx->stream>>>(
-                                           v, ctx->isect_state, ctx->isect_N));
-      RPBA_KERNEL(ctx, "k_isect_point", k_isect_point<double><<<nblk(ctx->N, 256), 256, 0, ctx->stream>>>(
-                                            v, ctx->isect_state, ctx->isect_iter, ctx->isect_N, maxit, tol, px_tol,
-                                            ctx->opt.cond_max, it == maxit - 1));
-    }
+                                            v, list, n, mask, tp_copies && tp_only ? 1 : 0, ctx->isect_state,
+                                            ctx->isect_iter, ctx->opt.isect_max_iter, ctx->opt.isect_tol,
+                                            ctx->opt.isect_px_tol, ctx->opt.cond_max));
+  } else if (n) {
+    if (ctx->has_winv && ctx->cd == 8) RPBA_TRY((isect_fp64<true, 8>(ctx, v, list, n, mask)));
+    else if (ctx->has_winv) RPBA_TRY((isect_fp64<true, 6>(ctx, v, list, n, mask)));
+    else if (ctx->cd == 8) RPBA_TRY((isect_fp64<false, 8>(ctx, v, list, n, mask)));
+    else RPBA_TRY((isect_fp64<false, 6>(ctx, v, list, n, mask)));
   }
   if (!n_dropped) return RPBA_OK;  // no count wanted: no host synchronisation
   RPBA_CUDA(cudaMemsetAsync(ctx->counters, 0, 4 * sizeof(int), ctx->stream));

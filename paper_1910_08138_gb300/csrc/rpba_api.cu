@@ -640,7 +640,13 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
   size_t rs = ctx->opt.precision == 1 ? sizeof(float) : sizeof(double);
   RPBA_TRY(dev_alloc(ctx, &ctx->Ninv, 6 * (size_t)P * rs));
   RPBA_TRY(dev_alloc(ctx, &ctx->gX, 3 * (size_t)P * rs));
-  RPBA_TRY(alloc_n(ctx, &ctx->isect_N, 10 * (size_t)P));
+  {
+    std::vector<int> ptr(N + 1, 0);
+    for (int j = 0; j < N; j++) ptr[j + 1] = ptr[j] + ctx->h_pt_nobs[j];
+    RPBA_TRY(upload(ctx, &ctx->pt_obs_ptr, ptr.data(), ptr.size()));
+    RPBA_TRY(alloc_n(ctx, &ctx->pt_obs, (size_t)K));
+    RPBA_TRY(point_obs_setup(ctx));
+  }
   RPBA_TRY(alloc_n(ctx, &ctx->isect_state, (size_t)N));
   RPBA_TRY(alloc_n(ctx, &ctx->isect_iter, (size_t)N));
   RPBA_TRY(upload(ctx, &ctx->obs_cam, ocam.data(), (size_t)K));

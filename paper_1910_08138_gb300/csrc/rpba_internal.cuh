@@ -289,7 +289,8 @@ struct Ctx {
   double *Xl = nullptr, *Xlt = nullptr, *Wl = nullptr, *inst_cost = nullptr;
   void *Ninv = nullptr, *gX = nullptr;  // compute precision
   // intersection scratch
-  double *isect_N = nullptr;  // P x 9 (sym3 + gradient)
+  // the observations by point, for the FP64 intersection (k_point_obs)
+  int *pt_obs_ptr = nullptr, *pt_obs = nullptr;
   int *isect_state = nullptr; // N: 0 idle, 1 running, 2 converged, 3 failed
   int *isect_iter = nullptr;
   // observations
@@ -556,6 +557,8 @@ rpba_status cost_sigma0_launch(Ctx *ctx);
 #define RPBA_CAM_STAGE_BYTES 144
 #define RPBA_COST_STAGE_MAX_SMEM (96 * 1024)  // 682 cameras: local indices fit 16 bits
 rpba_status cost_groups_setup(Ctx *ctx);
+// the observations by point, from the instance lists
+rpba_status point_obs_setup(Ctx *ctx);
 // the camera-major copies (FP32 form), from the observation-order arrays
 rpba_status camera_major_setup(Ctx *ctx);
 void sigma0_finish(const Ctx *ctx, double *sigma0, double *rms, long long *n_obs, long long *n_points);
