@@ -396,7 +396,10 @@ rpba_status rpba_profile_enable(rpba_ctx *ctx, int32_t enable);
 rpba_status rpba_profile_select(rpba_ctx *ctx, const char *kernel);
 /* Kernel launches since the last rpba_profile_enable, per kernel name (names:
  * max_kernels slots of 48 chars), their summed event time in ms (0 when
- * timing was off), the number of distinct kernels and of launches. */
+ * timing was off), the number of distinct kernels and of launches.
+ * The phases of k_pcg_solve (the FP32 form's CG loop in one kernel) are listed
+ * under the names of the kernels that run them one by one, with how often they
+ * ran and without a time; they are not among the launches of *total_launches. */
 rpba_status rpba_profile_read(rpba_ctx *ctx, int32_t max_kernels, char *names, double *ms,
                               int64_t *launches, int32_t *n_kernels, int64_t *total_launches);
 

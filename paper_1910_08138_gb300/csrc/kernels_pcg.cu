@@ -31,6 +31,7 @@
 // RCS; at the benchmark sizes two stages reach 1e-8. The CG steps thus read
 // half the bytes and run no float-float arithmetic, and the stopping test is
 // on the float-float true residual, not on a recurrence.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -211,26 +212,43 @@ __global__ void __launch_bounds__(256) k_pcg_split(const double *__restrict__ S,
 // S_hi p (and their total) is below np max|S_hi| max|p| < 2^61 2^-s, so the
 // partials scaled by 2^s fit 64-bit integers, whose sums are exact and do not
 // depend on the order of the atomics. Computed from the exponents alone.
-__device__ inline int fixed_exp(int np, float smax, float pmax) {
-  if (!(smax > 0.f) || !(pmax > 0.f) || isinf(smax) || isinf(pmax)) return 0;
-  int e1, e2, e3;
-  frexpf((float)np, &e1);
-  frexpf(smax, &e2);
-  frexpf(pmax, &e3);
-  return 61 - (e1 + e2 + e3);
+__device__ __forceinline__ int float_exp(float x) {  // frexp's exponent of a positive finite x
+  int e = (int)(__float_as_uint(x) >> 23);
+  if (e == 0) frexpf(x, &e);
+  else e -= 126;
+  return e;
 }
+__device__ __forceinline__ int fixed_exp(int np, float smax, float pmax) {
+  if (!(smax > 0.f) || !(pmax > 0.f) || isinf(smax) || isinf(pmax)) return 0;
+  return 61 - ((32 - __clz(np)) + float_exp(smax) + float_exp(pmax));
+}
+
+// x 2^e as scalbnf rounds it, by two exact factors; e is the same for many x.
+// A first product that underflows belongs to a value whose end result is zero
+// in the fixed-point format; beyond |e| = 252 scalbnf itself.
+struct Pow2 {
+  float a, b;
+  int e;
+  __device__ __forceinline__ explicit Pow2(int ex) : e(ex) {
+    int h = ex / 2;
+    bool in = abs(ex) <= 252;
+    a = in ? __int_as_float((127 + h) << 23) : 0.f;
+    b = in ? __int_as_float((127 + ex - h) << 23) : 0.f;
+  }
+  __device__ __forceinline__ float mul(float x) const { return a != 0.f ? __fmul_rn(__fmul_rn(x, a), b) : scalbnf(x, e); }
+};
 
 // FP32 form, refinement residual: q += S (X + dx) in float-float over the
 // lower tiles of the active sub-blocks (X float-float, dx the FP32 solution of
 // the stage just ended), summed over the tiles with FP64 atomics. One warp per
 // tile, the warps striding over the tile table (as k_pcg_symv32): lane c reads
-// column c's hi and lo words one row at a time, accumulates the transposed
-// product in float-float and keeps the 32 row terms (hi, lo); a transposing
-// butterfly of float-float additions leaves row r's sum in lane r.
+// column c's hi and lo words one row at a time and accumulates the transposed
+// product in float-float; a transposing butterfly of float-float additions over
+// the 32 row terms (hi, lo) leaves row r's sum in lane r.
 #define SYMV_THREADS 256
-__device__ __forceinline__ float2 warp_transpose_sum_ff(float (&th)[PT], float (&tl)[PT], int lane) {
+__device__ __forceinline__ float2 warp_transpose_sum_ff(float (&th)[PT / 2], float (&tl)[PT / 2], int lane) {
 #pragma unroll
-  for (int o = PT / 2; o >= 1; o >>= 1) {
+  for (int o = PT / 4; o >= 1; o >>= 1) {
     bool up = (lane & o) != 0;
 #pragma unroll
     for (int i = 0; i < o; i++) {
@@ -245,50 +263,96 @@ __device__ __forceinline__ float2 warp_transpose_sum_ff(float (&th)[PT], float (
   return make_float2(th[0], tl[0]);
 }
 
+// one tile (one warp) at (a, b) of a sub-block: Shi and Slo from its first
+// entry, X, dx and q from its first unknown. HOLD keeps the whole tile in
+// registers between the two products; otherwise (k_pcg_solve, 64 registers) the
+// row terms come from a second pass over the tile, then in the L1.
+template <bool HOLD>
+__device__ __forceinline__ void symv_ff_tile(const float *__restrict__ Shi, const float *__restrict__ Slo, int np,
+                                             int a, int b, const float2 *X, const float *dx, double *q, int lane) {
+  const size_t base = (size_t)(a * PT) * np + b * PT + lane;
+  Shi += base;
+  Slo += base;
+  float2 pI = ff_add(__ldcg(X + a * PT + lane), make_float2(__ldcg(dx + a * PT + lane), 0.f));
+  float2 pJ = ff_add(__ldcg(X + b * PT + lane), make_float2(__ldcg(dx + b * PT + lane), 0.f));
+  const bool diag = a == b;
+  constexpr int KEEP = HOLD ? PT : 8;
+  float hi[KEEP], lo[KEEP];
+  auto load = [&](int r0) {  // rows r0 .. of the lane's column; on a diagonal tile row r's columns 0 .. r
+#pragma unroll
+    for (int k = 0; k < KEEP; k++) {
+      hi[k] = __ldg(Shi + (size_t)(r0 + k) * np);
+      lo[k] = __ldg(Slo + (size_t)(r0 + k) * np);
+    }
+    if (diag)
+#pragma unroll
+      for (int k = 0; k < KEEP; k++)
+        if (lane > r0 + k) hi[k] = lo[k] = 0.f;
+  };
+  float2 col = make_float2(0.f, 0.f);
+#pragma unroll(HOLD ? 1 : 4)
+  for (int r0 = 0; r0 < PT; r0 += KEEP) {
+    load(r0);
+#pragma unroll
+    for (int k = 0; k < KEEP; k++) {
+      int r = r0 + k;
+      float2 pr = make_float2(__shfl_sync(0xffffffffu, pI.x, r), __shfl_sync(0xffffffffu, pI.y, r));
+      if (!diag || lane < r) col = ff_add(col, ff_mul(make_float2(hi[k], lo[k]), pr));
+    }
+  }
+  // the row terms, rows i and i + 16 together: the butterfly's first exchange
+  // halves what is kept
+  float th[PT / 2], tl[PT / 2];
+  const bool up16 = (lane & 16) != 0;
+  auto exchange = [&](int i, float2 mu, float2 mv) {
+    float2 u = ff_mul(mu, pJ), v = ff_mul(mv, pJ);
+    float2 send = up16 ? u : v, keep = up16 ? v : u;
+    float2 t = ff_add(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, 16),
+                                        __shfl_xor_sync(0xffffffffu, send.y, 16)));
+    th[i] = t.x;
+    tl[i] = t.y;
+  };
+  if constexpr (HOLD) {
+#pragma unroll
+    for (int i = 0; i < PT / 2; i++) exchange(i, make_float2(hi[i], lo[i]), make_float2(hi[i + 16], lo[i + 16]));
+  } else {
+#pragma unroll
+    for (int i0 = 0; i0 < PT / 2; i0 += 4) {
+      float2 u[4], v[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        int i = i0 + k;
+        u[k] = make_float2(__ldg(Shi + (size_t)i * np), __ldg(Slo + (size_t)i * np));
+        v[k] = make_float2(__ldg(Shi + (size_t)(i + 16) * np), __ldg(Slo + (size_t)(i + 16) * np));
+        if (diag && lane > i) u[k] = make_float2(0.f, 0.f);
+        if (diag && lane > i + 16) v[k] = make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) exchange(i0 + k, u[k], v[k]);
+    }
+  }
+  float2 row = warp_transpose_sum_ff(th, tl, lane);
+  if (!diag) {
+    atomicAdd(q + a * PT + lane, ff_to_double(row));
+    atomicAdd(q + b * PT + lane, ff_to_double(col));
+  } else {
+    atomicAdd(q + a * PT + lane, ff_to_double(ff_add(row, col)));
+  }
+}
+
 __global__ void __launch_bounds__(SYMV_THREADS) k_pcg_symv_ff(const float *__restrict__ Shi,
                                                               const float *__restrict__ Slo, const long long *S_off,
                                                               const int *npad, const int *voff, const int *act,
                                                               const int2 *__restrict__ tile_map, int tiles,
-                                                              const float2 *__restrict__ X,
-                                                              const float *__restrict__ dx, double *q) {
+                                                              const float2 *X, const float *dx, double *q) {
   int lane = threadIdx.x & 31;
   int nw = gridDim.x * (SYMV_THREADS / 32);
   for (int idx = blockIdx.x * (SYMV_THREADS / 32) + (threadIdx.x >> 5); idx < tiles; idx += nw) {
     int2 tm = tile_map[idx];
-    int l = tm.x, a = tm.y >> 16, b = tm.y & 0xffff;
+    int l = tm.x;
     if (!act[l]) continue;  // the same for the whole warp
-    int np = npad[l];
-    size_t base = (size_t)S_off[l] + (size_t)(a * PT) * np + b * PT + lane;
-    const float2 *Xl = X + voff[l];
-    const float *dxl = dx + voff[l];
-    float2 pI = ff_add(Xl[a * PT + lane], make_float2(dxl[a * PT + lane], 0.f));
-    float2 pJ = ff_add(Xl[b * PT + lane], make_float2(dxl[b * PT + lane], 0.f));
-    float th[PT], tl[PT];
-#pragma unroll
-    for (int r = 0; r < PT; r++) {
-      th[r] = __ldg(Shi + base + (size_t)r * np);
-      tl[r] = __ldg(Slo + base + (size_t)r * np);
-    }
-    float2 col = make_float2(0.f, 0.f);
-    const bool diag = a == b;
-#pragma unroll
-    for (int r = 0; r < PT; r++) {
-      float2 m = make_float2(th[r], tl[r]);
-      if (diag && lane > r) m = make_float2(0.f, 0.f);  // row r, columns 0 .. r
-      float2 pr = make_float2(__shfl_sync(0xffffffffu, pI.x, r), __shfl_sync(0xffffffffu, pI.y, r));
-      if (!diag || lane < r) col = ff_add(col, ff_mul(m, pr));
-      float2 t = ff_mul(m, pJ);
-      th[r] = t.x;
-      tl[r] = t.y;
-    }
-    float2 row = warp_transpose_sum_ff(th, tl, lane);
-    double *ql = q + voff[l];
-    if (!diag) {
-      atomicAdd(ql + a * PT + lane, ff_to_double(row));
-      atomicAdd(ql + b * PT + lane, ff_to_double(col));
-    } else {
-      atomicAdd(ql + a * PT + lane, ff_to_double(ff_add(row, col)));
-    }
+    symv_ff_tile<true>(Shi + S_off[l], Slo + S_off[l], npad[l], tm.y >> 16, tm.y & 0xffff, X + voff[l], dx + voff[l],
+                 q + voff[l], lane);
   }
 }
 
@@ -320,21 +384,18 @@ __device__ __forceinline__ float warp_transpose_sum(float (&t)[PT], int lane) {
 // sums of a lane (formed in a fixed order) are added to q as 64-bit fixed-point
 // integers (scale 2^s, fixed_exp), so q does not depend on the order of the
 // atomics and two runs give the same CG iterates.
-// one tile (one warp): tm = (sub-block, a << 16 | b)
-__device__ __forceinline__ void symv32_tile(const float *__restrict__ Shi, const long long *S_off, const int *npad,
-                                            const int *voff, const int *live, int2 tm,
-                                            const float *__restrict__ s32, const float *__restrict__ p,
-                                            unsigned long long *q, int lane) {
-  int l = tm.x, a = tm.y >> 16, b = tm.y & 0xffff;
-  if (!live[l]) return;
-  int np = npad[l];
-  int sc = (int)s32[PCG_S32 * l + S32_QEXP];
-  const float *A = Shi + S_off[l] + (size_t)(a * PT) * np + b * PT + lane;
-  const float *pl = p + voff[l];
-  float pIc = pl[a * PT + lane], pJc = pl[b * PT + lane];
-  float t[PT];
+// one tile (one warp) at (a, b) of a sub-block: A from its first entry, p and
+// q from its first unknown, up the scale of the fixed-point product
+__device__ __forceinline__ void symv32_load(const float *__restrict__ A, int np, int a, int b, int lane,
+                                            float (&t)[PT]) {
+  A += (size_t)(a * PT) * np + b * PT + lane;
 #pragma unroll
   for (int r = 0; r < PT; r++) t[r] = __ldg(A + (size_t)r * np);
+}
+
+__device__ __forceinline__ void symv32_product(float (&t)[PT], int a, int b, const Pow2 &up, const float *p,
+                                               unsigned long long *q, int lane) {
+  float pIc = __ldcg(p + a * PT + lane), pJc = __ldcg(p + b * PT + lane);
   float col = 0.f;
   if (a != b) {
 #pragma unroll
@@ -351,14 +412,20 @@ __device__ __forceinline__ void symv32_tile(const float *__restrict__ Shi, const
     }
   }
   float row = warp_transpose_sum(t, lane);
-  unsigned long long *ql = q + voff[l];
-  long long vr = __float2ll_rn(scalbnf(row, sc)), vc = __float2ll_rn(scalbnf(col, sc));
+  long long vr = __float2ll_rn(up.mul(row)), vc = __float2ll_rn(up.mul(col));
   if (a != b) {
-    atomicAdd(ql + a * PT + lane, (unsigned long long)vr);
-    atomicAdd(ql + b * PT + lane, (unsigned long long)vc);
+    atomicAdd(q + a * PT + lane, (unsigned long long)vr);
+    atomicAdd(q + b * PT + lane, (unsigned long long)vc);
   } else {
-    atomicAdd(ql + a * PT + lane, (unsigned long long)(vr + vc));
+    atomicAdd(q + a * PT + lane, (unsigned long long)(vr + vc));
   }
+}
+
+__device__ __forceinline__ void symv32_tile(const float *__restrict__ A, int np, int a, int b, const Pow2 &up,
+                                            const float *p, unsigned long long *q, int lane) {
+  float t[PT];
+  symv32_load(A, np, a, b, lane, t);
+  symv32_product(t, a, b, up, p, q, lane);
 }
 
 // The warps stride over the tiles (a grid of a few CTAs per SM), each tile's
@@ -368,73 +435,79 @@ __global__ void __launch_bounds__(32 * SYMV32_WARPS) k_pcg_symv32(const float *_
                                                                   const long long *S_off, const int *npad,
                                                                   const int *voff, const int *live,
                                                                   const int2 *__restrict__ tile_map, int tiles,
-                                                                  const float *__restrict__ s32,
-                                                                  const float *__restrict__ p,
+                                                                  const float *__restrict__ s32, const float *p,
                                                                   unsigned long long *q) {
   int lane = threadIdx.x & 31;
   int nw = gridDim.x * SYMV32_WARPS;
-  for (int idx = blockIdx.x * SYMV32_WARPS + (threadIdx.x >> 5); idx < tiles; idx += nw)
-    symv32_tile(Shi, S_off, npad, voff, live, tile_map[idx], s32, p, q, lane);
+  for (int idx = blockIdx.x * SYMV32_WARPS + (threadIdx.x >> 5); idx < tiles; idx += nw) {
+    int2 tm = tile_map[idx];
+    int l = tm.x;
+    if (!live[l]) continue;  // the same for the whole warp
+    symv32_tile(Shi + S_off[l], npad[l], tm.y >> 16, tm.y & 0xffff, Pow2((int)s32[PCG_S32 * l + S32_QEXP]),
+                p + voff[l], q + voff[l], lane);
+  }
 }
 
 // four CTAs of eight warps per SM (152 SMs), or one warp per tile if fewer
 static inline int symv32_grid(int tiles) { return std::max(1, std::min(nblk(tiles, SYMV32_WARPS), 4 * 152)); }
 
 // q[e] (fixed point, scale 2^s) as a float
-__device__ __forceinline__ float fixed_to_float(unsigned long long v, int sc) {
-  return scalbnf(__ll2float_rn((long long)v), -sc);
+__device__ __forceinline__ float fixed_to_float(unsigned long long v, const Pow2 &down) {
+  return down.mul(__ll2float_rn((long long)v));
 }
 
-// FP32 sums of NV values over the CTA; every thread gets the totals
-template <int NV>
-__device__ inline void f_cta_sum(float (&v)[NV], float (&out)[NV]) {
-  __shared__ float sh[NV][32];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; k++) {
-    float x = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[k][wid] = x;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; k++) {
-    float s = 0.f;
-    for (int w = 0; w < nw; w++) s += sh[k][w];
-    out[k] = s;
-  }
-  __syncthreads();
-}
+// barrier of the PCG_THREADS threads that do a step's or a stage's vector part
+// (all of their kernel's, or the first of a wider CTA)
+__device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, %0;" ::"n"(PCG_THREADS) : "memory"); }
 
-
-// FP32 sums of NV values and the maximum of one more over the CTA; every
-// thread gets the results
+// FP32 sums of NV values and the maximum of one more over these threads; each
+// gets the results. The scratch sh (one per call site) is written again
+// only after a later barrier of the CTA.
 template <int NV>
-__device__ inline void f_cta_sum_max(float (&v)[NV], float m, float (&out)[NV], float &mout) {
-  __shared__ float sh[NV + 1][32];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ void f_cta_sum_max(float (&v)[NV], float m, float (&out)[NV], float &mout,
+                                              float (&sh)[NV + 1][PCG_THREADS / 32]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < NV; k++) {
-    float x = v[k];
+  for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[k][wid] = x;
+    for (int k = 0; k < NV; k++) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   }
+  if (lane == 0) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) sh[NV][wid] = m;
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; k++) {
-    float t = 0.f;
-    for (int w = 0; w < nw; w++) t += sh[k][w];
-    out[k] = t;
+    for (int k = 0; k < NV; k++) sh[k][wid] = v[k];
+    sh[NV][wid] = m;
   }
+  step_sync();
   float mm = 0.f;
-  for (int w = 0; w < nw; w++) mm = fmaxf(mm, sh[NV][w]);
+#pragma unroll
+  for (int k = 0; k < NV; k++) out[k] = 0.f;
+#pragma unroll
+  for (int w = 0; w < PCG_THREADS / 32; w++) {
+#pragma unroll
+    for (int k = 0; k < NV; k++) out[k] += sh[k][w];
+    mm = fmaxf(mm, sh[NV][w]);
+  }
   mout = mm;
-  __syncthreads();
+}
+
+// FP64 sums of two values over the same threads, in the order of cta_sum
+__device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
+  __shared__ double sh[2][PCG_THREADS / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int e = 0; e < 2; e++) {
+    double x = v[e];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) sh[e][wid] = x;
+  }
+  step_sync();
+#pragma unroll
+  for (int e = 0; e < 2; e++) {
+    double s = 0.0;
+    for (int w = 0; w < PCG_THREADS / 32; w++) s += sh[e][w];
+    out[e] = s;
+  }
 }
 
 // FP32 form: start of a refinement stage, one CTA per active sub-block.
@@ -442,20 +515,19 @@ __device__ inline void f_cta_sum_max(float (&v)[NV], float m, float (&out)[NV], 
 // X += x, the FP32 solution of the stage just ended, and R = y - q with
 // q = S X from k_pcg_symv_ff (q is zeroed once read). The solve of the
 // sub-block ends when ||R|| <= tol ||y||, when a stage has not halved ||R||,
-// after max_stage stages, or at the CG step cap (final set, or the device
-// loop's step count loop_cnt[0] at max_iter);
+// after max_stage stages, or at the CG step cap (fin: the device loop's step
+// count loop_cnt[0] at max_iter, or the host loop's last stage);
 // otherwise the FP32 CG restarts on S_hi d = R rounded to FP32: x = 0,
 // z = M^-1 r, p = z, stopping at ||r|| <= max(tol_in, 0.3 tol ||y|| / ||R||)
 // ||R||. st[4l + 2] is the relative true residual ||R|| / ||y||.
+// Returns (uniformly) whether the CG restarts.
 template <int CD>
-__global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
-    int first, int final_stage, const int *loop_cnt, int max_iter, const int *run, const int *fail,
-    const int *sub_cam_ptr, const int *voff,
+__device__ bool pcg_stage_body(
+    int first, bool fin, int l, const int *run, const int *fail, const int *sub_cam_ptr, const int *voff,
     const int *npad, const float *__restrict__ Minv32, const double *__restrict__ y, double *qd, float2 *X,
     float *x, float *r, float *z, float *p, unsigned long long *q, double *st, float *s32, int *act, int *live,
     double tol, double tol_in, int max_stage) {
   __shared__ int stop;
-  int l = blockIdx.x;
   int stage;
   if (first) {
     int ok = run[l] && !fail[l];
@@ -466,17 +538,17 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
       st[4 * l + 2] = ok ? 1.0 : 0.0;
       s32[PCG_S32 * l + S32_STAGES] = 0.f;
     }
-    if (!ok) return;
+    if (!ok) return false;
     stage = 0;
   } else {
     stage = act[l];
-    if (!stage) return;
+    if (!stage) return false;
   }
   int g0 = sub_cam_ptr[l], ncam = sub_cam_ptr[l + 1] - g0;
   int n = CD * ncam, o = voff[l], np = npad[l];
   float rr = 0.f;             // ||R||^2: FP32 terms and per-thread sums, FP64 across the CTA
   double v[2] = {0.0, 0.0};  // ||R||^2, ||y||^2
-  for (int e = threadIdx.x; e < np; e += blockDim.x) {
+  for (int e = threadIdx.x; e < np; e += PCG_THREADS) {
     float re = 0.f;
     if (e < n) {
       float2 yf = ff_split_bits(y[o + e]);
@@ -486,7 +558,7 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
         v[1] += y[o + e] * y[o + e];
       } else {
         X[o + e] = ff_add(X[o + e], make_float2(x[o + e], 0.f));
-        float2 qf = ff_split_bits(qd[o + e]);
+        float2 qf = ff_split_bits(__ldcg(qd + o + e));
         R = ff_add(yf, make_float2(-qf.x, -qf.y));
       }
       rr = __fmaf_rn(R.x, R.x, rr);
@@ -503,7 +575,7 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
   }
   v[0] = f2d(rr);
   double s[2];
-  cta_sum<2>(v, s);  // its barriers also order the r writes before the reads below
+  stage_sum2(v, s);  // its barrier also orders the r writes before the reads below
   if (threadIdx.x == 0) {
     double ny = first ? sqrt(s[1]) : st[4 * l + 1];
     double nr = sqrt(s[0]);
@@ -511,7 +583,6 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
     if (first) st[4 * l + 1] = ny;
     st[4 * l + 2] = rel;
     float *w = s32 + PCG_S32 * l;
-    bool fin = final_stage || (loop_cnt && loop_cnt[0] >= max_iter);
     bool done = !(ny > 0.0) || rel <= tol || fin || stage >= max_stage ||
                 (!first && !(rel <= 0.5 * (double)w[S32_PREV]));
     if (done) {
@@ -527,10 +598,10 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
     }
     stop = done;
   }
-  __syncthreads();
-  if (stop) return;
+  step_sync();
+  if (stop) return false;
   float rz = 0.f, zmax = 0.f;
-  for (int c = threadIdx.x; c < ncam; c += blockDim.x) {
+  for (int c = threadIdx.x; c < ncam; c += PCG_THREADS) {
     const float *Mi = Minv32 + CD * CD * (size_t)(g0 + c);
     const float *rc = r + o + CD * c;
     float rl[CD];
@@ -547,14 +618,26 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
       zmax = fmaxf(zmax, fabsf(t));
     }
   }
+  __shared__ float sh_rz[2][PCG_THREADS / 32];
   float v1[1] = {rz}, t1[1], pmax;
-  f_cta_sum_max<1>(v1, zmax, t1, pmax);
+  f_cta_sum_max<1>(v1, zmax, t1, pmax, sh_rz);
   if (threadIdx.x == 0) {
     float *w = s32 + PCG_S32 * l;
     w[S32_RZ] = t1[0];
     w[S32_PMAX] = pmax;
     w[S32_QEXP] = (float)fixed_exp(np, w[S32_SMAX], pmax);
   }
+  return true;
+}
+
+template <int CD>
+__global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
+    int first, int final_stage, const int *loop_cnt, int max_iter, const int *run, const int *fail,
+    const int *sub_cam_ptr, const int *voff, const int *npad, const float *__restrict__ Minv32,
+    const double *__restrict__ y, double *qd, float2 *X, float *x, float *r, float *z, float *p,
+    unsigned long long *q, double *st, float *s32, int *act, int *live, double tol, double tol_in, int max_stage) {
+  pcg_stage_body<CD>(first, final_stage || (loop_cnt && loop_cnt[0] >= max_iter), blockIdx.x, run, fail, sub_cam_ptr, voff, npad, Minv32, y, qd, X, x, r,
+                     z, p, q, st, s32, act, live, tol, tol_in, max_stage);
 }
 
 // FP32 form, inner CG step of a refinement stage (one CTA per live
@@ -562,10 +645,121 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
 // beta = r.z / rz, p = z + beta p; the stage ends when ||r|| <= tol_s ||r_0||.
 // FP32 throughout, block sums included (the stage needs ~1e-4 of its right-hand
 // side; the refinement's float-float residual corrects the rest). Each thread
-// loads all of its elements at once (up to PCGF_PER) so that each phase waits
-// for one memory latency; r and z pass between the phases in shared memory;
-// q is zeroed once read.
+// loads all of its product's elements at once (up to PCGF_PER); q is zeroed
+// once read.
 #define PCGF_PER 8
+// a stage's scalars, the same in every thread of the CTA
+struct CgState {
+  float rz, rn0, tol, pmax;
+  int sc;
+};
+
+__device__ __forceinline__ CgState cg_load(const float *w) {
+  return {w[S32_RZ], w[S32_RN0], w[S32_TOL], w[S32_PMAX], (int)w[S32_QEXP]};
+}
+
+// one step on the vectors in shared memory (x, r, z, p, n floats each, one
+// after the other); the new p goes to memory too, for the next product. Mi:
+// the sub-block's inverse camera blocks. The chain of its phases is what a CG
+// step costs, so it keeps to two barriers and two reductions of the CTA.
+// 0: breakdown, 1: the stage's tolerance is reached, 2: go on
+template <int CD>
+__device__ __forceinline__ int cg_step_body(int ncam, int np, float smax, const float *Mi, unsigned long long *q,
+                                            float *p_out, float *vec, CgState &s) {
+  __shared__ float sh_pq[2][PCG_THREADS / 32], sh_rr[3][PCG_THREADS / 32];
+  const int n = CD * ncam;
+  float *xs = vec, *rs = vec + n, *zs = vec + 2 * n, *ps = vec + 3 * n;
+  const int nk = (n + PCG_THREADS - 1) / PCG_THREADS;
+  unsigned long long qi[PCGF_PER];
+#pragma unroll
+  for (int k = 0; k < PCGF_PER; k++)
+    if (k < nk) {
+      int e = threadIdx.x + k * PCG_THREADS;
+      qi[k] = e < n ? __ldcg(q + e) : 0ull;
+    }
+  const Pow2 down(-s.sc);
+  float pq = 0.f;
+#pragma unroll
+  for (int k = 0; k < PCGF_PER; k++)
+    if (k < nk) {
+      int e = threadIdx.x + k * PCG_THREADS;
+      float qe = fixed_to_float(qi[k], down);
+      if (e < n) {
+        q[e] = 0ull;
+        zs[e] = qe;  // until z is formed
+        pq = __fmaf_rn(ps[e], qe, pq);
+      }
+    }
+  float v1[1] = {pq}, t1[1], unused;
+  f_cta_sum_max<1>(v1, 0.f, t1, unused, sh_pq);
+  if (!(t1[0] > 0.f)) return 0;  // breakdown: the stage keeps its current iterate
+  float alpha = s.rz / t1[0];
+  float rr = 0.f;
+  for (int e = threadIdx.x; e < n; e += PCG_THREADS) {
+    xs[e] = __fmaf_rn(alpha, ps[e], xs[e]);
+    float re = __fmaf_rn(-alpha, zs[e], rs[e]);
+    rs[e] = re;
+    rr = __fmaf_rn(re, re, rr);
+  }
+  step_sync();
+  float rz = 0.f, zmax = 0.f;
+  for (int c = threadIdx.x; c < ncam; c += PCG_THREADS) {
+    const float4 *mc = reinterpret_cast<const float4 *>(Mi + CD * CD * c);
+    float rl[CD];
+#pragma unroll
+    for (int b = 0; b < CD; b++) rl[b] = rs[CD * c + b];
+    float m[CD * CD];
+#pragma unroll
+    for (int k = 0; k < CD * CD / 4; k++) {
+      float4 u = mc[k];
+      m[4 * k] = u.x; m[4 * k + 1] = u.y; m[4 * k + 2] = u.z; m[4 * k + 3] = u.w;
+    }
+#pragma unroll
+    for (int a = 0; a < CD; a++) {
+      float t = 0.f;
+#pragma unroll
+      for (int b = 0; b < CD; b++) t = __fmaf_rn(m[CD * a + b], rl[b], t);
+      zs[CD * c + a] = t;
+      rz = __fmaf_rn(rl[a], t, rz);
+      zmax = fmaxf(zmax, fabsf(t));
+    }
+  }
+  float v2[2] = {rr, rz}, t2[2], zm;
+  f_cta_sum_max<2>(v2, zmax, t2, zm, sh_rr);  // its barrier also orders the z writes before the reads below
+  float beta = t2[1] / s.rz;
+  s.rz = t2[1];
+  for (int e = threadIdx.x; e < n; e += PCG_THREADS) {
+    float pn = __fmaf_rn(beta, ps[e], zs[e]);
+    ps[e] = pn;
+    p_out[e] = pn;
+  }
+  // max |z + beta p| <= max |z| + |beta| max |p|: the next product's scale
+  s.pmax = zm + fabsf(beta) * s.pmax;
+  s.sc = fixed_exp(np, smax, s.pmax);
+  return sqrtf(t2[0]) <= s.tol * s.rn0 ? 1 : 2;
+}
+
+// the vectors of a sub-block into shared memory (z needs no start value)
+__device__ __forceinline__ void cg_load_vectors(int n, const float *x, const float *r, const float *p, float *vec) {
+  for (int e = threadIdx.x; e < n; e += PCG_THREADS) {  // each thread uses only what it loads, until the barriers
+    vec[e] = x[e];
+    vec[n + e] = r[e];
+    vec[3 * n + e] = p[e];
+  }
+}
+
+// M^-1 into shared memory behind the vectors (used after the step's barriers)
+template <int CD>
+__device__ __forceinline__ const float *cg_load_minv(int n, const float *minv, float *vec) {
+  float4 *ms = reinterpret_cast<float4 *>(vec + 4 * ((n + 3) & ~3));
+  for (int e = threadIdx.x; e < CD * n / 4; e += PCG_THREADS) ms[e] = __ldg(reinterpret_cast<const float4 *>(minv) + e);
+  return reinterpret_cast<const float *>(ms);
+}
+
+// The same step as a launch of its own. Everything comes from memory, so each
+// thread loads all it needs at once (M^-1 of its camera included) and keeps it
+// in registers: 9.2 us for 64 sub-blocks of 936 unknowns, 10.7 us with
+// cg_step_body on staged vectors.
 template <int CD>
 __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_ptr, const int *voff,
                                                             const float *__restrict__ Minv32,
@@ -573,15 +767,16 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
                                                             float *__restrict__ r, float *__restrict__ p,
                                                             unsigned long long *__restrict__ q, double *st,
                                                             float *s32, int *live) {
-  extern __shared__ float rzs[];  // r (n), then z (n)
+  extern __shared__ __align__(16) float vec[];  // r (n), then z (n)
+  __shared__ float sh_pq[2][PCG_THREADS / 32], sh_rr[3][PCG_THREADS / 32];
   int l = blockIdx.x;
   if (!live[l]) return;
   int g0 = sub_cam_ptr[l], ncam = sub_cam_ptr[l + 1] - g0;
   int n = CD * ncam, o = voff[l];
-  float *rs = rzs, *zs = rzs + n;
+  float *rs = vec, *zs = vec + n;
   float *w = s32 + PCG_S32 * l;
   float rz_old = w[S32_RZ], rn0 = w[S32_RN0], tol_s = w[S32_TOL], pmax_old = w[S32_PMAX];
-  int sc = (int)w[S32_QEXP];
+  const Pow2 down(-(int)w[S32_QEXP]);
   constexpr int M4 = CD * CD / 4;
   float m[CD * CD];
   int c0 = threadIdx.x;
@@ -597,7 +792,7 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
 #pragma unroll
   for (int k = 0; k < PCGF_PER; k++) {
     int e = threadIdx.x + k * PCG_THREADS;
-    if (e < n) { pv[k] = p[o + e]; xv[k] = x[o + e]; rv[k] = r[o + e]; qv[k] = fixed_to_float(q[o + e], sc); }
+    if (e < n) { pv[k] = p[o + e]; xv[k] = x[o + e]; rv[k] = r[o + e]; qv[k] = fixed_to_float(q[o + e], down); }
   }
   float pq = 0.f;
 #pragma unroll
@@ -608,8 +803,8 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
       pq = __fmaf_rn(pv[k], qv[k], pq);
     }
   }
-  float v1[1] = {pq}, t1[1];
-  f_cta_sum<1>(v1, t1);
+  float v1[1] = {pq}, t1[1], unused;
+  f_cta_sum_max<1>(v1, 0.f, t1, unused, sh_pq);
   if (!(t1[0] > 0.f)) {  // breakdown: the stage keeps its current iterate
     if (threadIdx.x == 0) live[l] = 0;
     return;
@@ -652,7 +847,7 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
     }
   }
   float v2[2] = {rr, rz}, t2[2], zm;
-  f_cta_sum_max<2>(v2, zmax, t2, zm);  // its barrier also orders the z writes before the reads below
+  f_cta_sum_max<2>(v2, zmax, t2, zm, sh_rr);  // its barrier also orders the z writes before the reads below
   float beta = t2[1] / rz_old;
   if (threadIdx.x == 0) {
     w[S32_RZ] = t2[1];
@@ -667,6 +862,135 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
   for (int k = 0; k < PCGF_PER; k++) {
     int e = threadIdx.x + k * PCG_THREADS;
     if (e < n) p[o + e] = __fmaf_rn(beta, pv[k], zs[e]);
+  }
+}
+
+// The whole loop of a solve in one launch: one thread block cluster per
+// sub-block runs the CG steps and the refinement stages that follow
+// k_pcg_stage's start. A step is a product over the sub-block's tiles by every
+// warp of the cluster (q by 64-bit fixed-point atomics, as k_pcg_symv32), a
+// cluster barrier, the vector part by CTA 0 (the arithmetic of k_pcg_step32),
+// which hands the others the continue flag and the product's exponent through
+// their shared memory, and a cluster barrier; likewise the stage's float-float
+// product and k_pcg_stage's part. All loops end by max_iter steps and
+// max_stage stages. What other CTAs write (p, q, X, x) is read past the L1.
+// The same iterates as the kernels launched one by one. As three graph nodes
+// in a conditional loop a step took about 14 us whatever its size, all
+// sub-blocks in lock step; here two sub-blocks of 150 unknowns take 4.2 us per
+// step (1.3 us the product, 1.3 us the vector part, the rest barriers; the
+// 50-camera call 2.33 -> 1.40 ms) and eight of 720 to 780 11 us (the
+// 1,000-camera call 1.89 -> 1.79 ms).
+// stage_steps: per stage the most CG steps any sub-block took (max_stage
+// entries), then the most stages.
+struct PcgSolve {
+  int max_iter, max_stage, minv_in_smem;
+  const int *sub_cam_ptr, *voff, *npad, *tile_ptr;
+  const long long *S_off;
+  const int2 *tile_map;
+  const float *Shi, *Slo, *Minv32;
+  const double *y;
+  double *qd;
+  float2 *X;
+  float *x, *r, *z, *p;
+  unsigned long long *q;
+  double *st;
+  float *s32;
+  int *act, *live, *stage_steps;
+  double tol, tol_in;
+};
+
+// RES: every warp has at most one tile, whose entries stay in its registers for
+// the whole solve. Else the tiles come from the L2 or memory every step, and
+// 32 warps per CTA hide a tile's chain (position, entries, p, butterfly: about
+// 3,000 cycles of latency for 300 instructions).
+template <int CD, int WARPS, bool RES>
+__global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) float vec[];  // CTA 0: x, r, z, p and M^-1 (when it fits) of the sub-block
+  __shared__ int ctl[2];  // CTA 0's decision: go on; the exponent of the next product
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
+  const int l = blockIdx.x / C;
+  if (!v.act[l]) return;  // uniform over the cluster
+  const int lane = threadIdx.x & 31, warp = rank * WARPS + (threadIdx.x >> 5), warps = C * WARPS;
+  const bool vector_part = rank == 0 && threadIdx.x < PCG_THREADS;
+  const int np = v.npad[l], o = v.voff[l], t0 = v.tile_ptr[l], nt = v.tile_ptr[l + 1] - t0;
+  const int g0 = v.sub_cam_ptr[l], ncam = v.sub_cam_ptr[l + 1] - g0, n = CD * ncam;
+  const float *Shi = v.Shi + v.S_off[l], *Slo = v.Slo + v.S_off[l];
+  float *w = v.s32 + PCG_S32 * l;
+  const float smax = w[S32_SMAX];
+  auto tell = [&](int go, int sc) {  // to every CTA of the cluster, ordered by the barrier that follows
+    if ((int)threadIdx.x < C) {
+      int *c = cluster.map_shared_rank(ctl, threadIdx.x);
+      c[0] = go;
+      c[1] = sc;
+    }
+  };
+  const float *minv = v.Minv32 + CD * CD * (size_t)g0;
+  if (vector_part && v.minv_in_smem) minv = cg_load_minv<CD>(n, minv, vec);
+  float mine[RES ? PT : 1];  // this warp's tile, its lane's column
+  int ab = 0;
+  if constexpr (RES) {
+    if (warp < nt) {
+      ab = v.tile_map[t0 + warp].y;
+      symv32_load(Shi, np, ab >> 16, ab & 0xffff, lane, mine);
+    }
+  }
+  int go = v.live[l], sc = (int)w[S32_QEXP], steps = 0, stages = 0;
+  while (go) {
+    CgState s = cg_load(w);
+    int in_stage = 0;
+    if (vector_part) cg_load_vectors(n, v.x + o, v.r + o, v.p + o, vec);
+    while (go) {
+      const Pow2 up(sc);
+      if constexpr (RES) {
+        if (warp < nt) {
+          float t[PT];
+#pragma unroll
+          for (int r = 0; r < PT; r++) t[r] = mine[r];
+          symv32_product(t, ab >> 16, ab & 0xffff, up, v.p + o, v.q + o, lane);
+        }
+      } else {
+        for (int t = warp; t < nt; t += warps) {
+          int pos = v.tile_map[t0 + t].y;
+          symv32_tile(Shi, np, pos >> 16, pos & 0xffff, up, v.p + o, v.q + o, lane);
+        }
+      }
+      cluster.sync();
+      if (vector_part) {
+        int res = cg_step_body<CD>(ncam, np, smax, minv, v.q + o, v.p + o, vec, s);
+        in_stage += res != 0;
+        const bool more = res == 2 && steps + in_stage < v.max_iter;
+        if (!more)  // the stage's solution, for the float-float product
+          for (int e = threadIdx.x; e < n; e += PCG_THREADS) v.x[o + e] = vec[e];
+        tell(more, s.sc);
+      }
+      cluster.sync();
+      go = ctl[0];
+      sc = ctl[1];
+    }
+    for (int t = warp; t < nt; t += warps) {
+      int pos = v.tile_map[t0 + t].y;
+      symv_ff_tile<RES>(Shi, Slo, np, pos >> 16, pos & 0xffff, v.X + o, v.x + o, v.qd + o, lane);
+    }
+    cluster.sync();
+    if (vector_part) {
+      steps += in_stage;
+      if (threadIdx.x == 0) {
+        v.st[4 * l + 3] = (double)steps;
+        atomicMax(v.stage_steps + stages, in_stage);
+        atomicMax(v.stage_steps + v.max_stage, stages + 1);
+      }
+      bool more = pcg_stage_body<CD>(0, steps >= v.max_iter, l, nullptr, nullptr, v.sub_cam_ptr, v.voff, v.npad,
+                                     v.Minv32, v.y, v.qd, v.X, v.x, v.r, v.z, v.p, v.q, v.st, v.s32, v.act, v.live,
+                                     v.tol, v.tol_in, v.max_stage);
+      step_sync();  // thread 0's words of w
+      tell(more, (int)w[S32_QEXP]);
+    }
+    stages++;
+    cluster.sync();
+    go = ctl[0];
+    sc = ctl[1];
   }
 }
 
@@ -1147,17 +1471,54 @@ __global__ void __launch_bounds__(256) k_pcg_cond(cudaGraphConditionalHandle h, 
   }
 }
 
+// the phases of k_pcg_solve as the profile lists them: the names of the kernels
+// that run them when launched one by one
+static const char *const kCgPhases[] = {"k_pcg_symv32", "k_pcg_step32", "k_pcg_cond"};
+static const char *const kStagePhases[] = {"k_pcg_symv_ff", "k_pcg_stage", "k_pcg_cond"};
+
 static bool pcg_loop_kernel(const std::string &n) {
-  return n == "k_pcg_symv32" || n == "k_pcg_step32" || n == "k_pcg_cond" || n == "k_pcg_symv_ff" ||
-         n == "k_pcg_stage";
+  for (const char *k : kCgPhases)
+    if (n == k) return true;
+  for (const char *k : kStagePhases)
+    if (n == k) return true;
+  return false;
 }
 
 bool pcg_device_loop(const Ctx *ctx) {
-  if (!ff_pcg(ctx) || ctx->pcg_no_device_loop || !ctx->pcg_body_stream[0] || !ctx->pcg_body_stream[1])
-    return false;
-  // conditional bodies take no event-record nodes: a loop kernel that is
-  // being timed runs in the host-driven loop
-  return !(ctx->prof_enabled && (ctx->prof_only.empty() || pcg_loop_kernel(ctx->prof_only)));
+  if (!ff_pcg(ctx) || ctx->pcg_no_device_loop) return false;
+  // neither form times a phase: conditional bodies take no event-record nodes,
+  // and k_pcg_solve's phases are no launches; a loop kernel that is being timed
+  // runs in the host-driven loop
+  return (ctx->pcg_fused || (ctx->pcg_body_stream[0] && ctx->pcg_body_stream[1])) &&
+         !(ctx->prof_enabled && (ctx->prof_only.empty() || pcg_loop_kernel(ctx->prof_only)));
+}
+
+// lock-step CG steps (per stage the slowest sub-block's) and stages of the last
+// solve of the device-driven loop, from its counters in pinned memory
+int pcg_loop_steps(const Ctx *ctx, int *stages) {
+  const int *c = ctx->h_pinned_counter + PCG_LOOP_COUNTERS;
+  int n = 0;
+  if (!ctx->pcg_fused) {
+    if (stages) *stages = c[1];
+    return c[0];
+  }
+  for (int k = 0; k < RPBA_PCG_MAX_STAGES; k++) n += c[k];
+  if (stages) *stages = c[RPBA_PCG_MAX_STAGES];
+  return std::min(n, ctx->opt.pcg_max_iter);
+}
+
+// after a solve by k_pcg_solve: its phases, as often as they ran (they are no
+// launches); after a graph with the conditional loop: its bodies' launches
+void pcg_loop_account(Ctx *ctx, const GraphRec *g) {
+  int stages, steps = pcg_loop_steps(ctx, &stages);
+  if (ctx->pcg_fused) {
+    for (const char *k : kCgPhases) ctx->launch_by_name[k] += steps;
+    for (const char *k : kStagePhases) ctx->launch_by_name[k] += stages;
+    return;
+  }
+  for (const char *k : g->loop_inner) ctx->launch_by_name[k] += steps;
+  for (const char *k : g->loop_outer) ctx->launch_by_name[k] += stages;
+  ctx->launches += (long long)steps * g->loop_inner.size() + (long long)stages * g->loop_outer.size();
 }
 
 // a while node after the work captured so far on st, with its handle; the
@@ -1262,11 +1623,87 @@ static rpba_status pcg_loop_device(Ctx *ctx) {
   return RPBA_OK;
 }
 
+typedef void (*PcgSolveKernel)(PcgSolve);
+static PcgSolveKernel pcg_solve_kernel(const Ctx *ctx) {
+  if (ctx->cd == 8) return ctx->pcg_res ? k_pcg_solve<8, 8, true> : k_pcg_solve<8, 32, false>;
+  return ctx->pcg_res ? k_pcg_solve<6, 8, true> : k_pcg_solve<6, 32, false>;
+}
+
+// k_pcg_solve or the loop of graph nodes: the nodes spread the products over
+// the whole chip, but a step costs three launches and the sub-blocks wait for
+// each other. One kernel is faster while an SM gets up to two tiles per warp:
+// eight sub-blocks of 750 unknowns (41 tiles per CTA) 1.79 against 1.89 ms per
+// call; beyond that its product, which is bound by the instructions of the
+// fewer SMs, loses: 64 sub-blocks of 936 (232 tiles per CTA) 4.80 against
+// 4.40 ms.
+#define PCG_FUSED_TILES 64
+// The shape of k_pcg_solve: CTAs per cluster C up to eight (the portable size)
+// while all clusters fit the chip at once (one CTA per SM, 152). The register
+// form, eight warps per CTA, when that gives one warp per tile of the largest
+// sub-block (up to 64 tiles, 320 unknowns); else 32 warps per CTA. M^-1 (cd
+// floats per unknown, else an L2 round trip of every step) goes to shared
+// memory beside the vectors while both fit 48 KB.
+rpba_status pcg_solve_setup(Ctx *ctx, int max_n) {
+  const int n4 = (std::max(max_n, 1) + 3) & ~3;
+  const long long tiles = (long long)ctx->max_tiles * (ctx->max_tiles + 1) / 2;
+  const size_t vec = (size_t)n4 * 4 * sizeof(float), minv = (size_t)n4 * ctx->cd * sizeof(float);
+  ctx->pcg_ff_smem = vec / 2;
+  ctx->pcg_minv_smem = vec + minv <= 48 * 1024 ? 1 : 0;
+  ctx->pcg_solve_smem = vec + (ctx->pcg_minv_smem ? minv : 0);
+  auto cluster = [&](int warps) {
+    int C = 8;
+    while (C > 1 && ((long long)(C - 1) * warps >= tiles || (long long)C * ctx->L > 152)) C--;
+    return C;
+  };
+  int C = cluster(8);
+  ctx->pcg_res = (long long)C * 8 >= tiles && (long long)C * ctx->L <= 152;
+  ctx->pcg_cluster = ctx->pcg_res ? C : cluster(32);
+  ctx->pcg_fused = (tiles + ctx->pcg_cluster - 1) / ctx->pcg_cluster <= PCG_FUSED_TILES &&
+                   (long long)ctx->pcg_cluster * ctx->L <= 152;
+  return RPBA_OK;
+}
+
+static rpba_status pcg_solve(Ctx *ctx, int *iters) {
+  cudaStream_t st = ctx->stream;
+  int *cnt = ctx->counters + PCG_LOOP_COUNTERS;
+  const size_t cnt_bytes = (RPBA_PCG_MAX_STAGES + 1) * sizeof(int);
+  RPBA_CUDA(cudaMemsetAsync(cnt, 0, cnt_bytes, st));
+  PcgSolve v{ctx->opt.pcg_max_iter, RPBA_PCG_MAX_STAGES, ctx->pcg_minv_smem, ctx->sub_cam_ptr, ctx->ycam_off,
+             ctx->npad, ctx->pcg_tiles, ctx->S_off, ctx->pcg_tile_map, ctx->pcg_Shi, ctx->pcg_Slo, ctx->pcg_Minv32,
+             ctx->y, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32, ctx->pcg_r32, ctx->pcg_z32, ctx->pcg_p32, ctx->pcg_qi,
+             ctx->pcg_st, ctx->pcg_s32, ctx->pcg_act, ctx->pcg_live, cnt, ctx->opt.pcg_tol, RPBA_PCG_INNER_TOL};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctx->pcg_cluster * ctx->L);
+  cfg.blockDim = dim3(ctx->pcg_res ? 8 * 32 : 32 * 32);
+  cfg.dynamicSmemBytes = ctx->pcg_solve_smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctx->pcg_cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (ctx->L) RPBA_KERNEL(ctx, "k_pcg_solve", RPBA_CUDA(cudaLaunchKernelEx(&cfg, pcg_solve_kernel(ctx), v)));
+  RPBA_CUDA(cudaMemcpyAsync(ctx->h_pinned_counter + PCG_LOOP_COUNTERS, cnt, cnt_bytes, cudaMemcpyDeviceToHost, st));
+  if (iters) *iters = 0;  // in a graph: known after the replay (pinned counters)
+  if (ctx->capture) {
+    ctx->capture->pcg_loop = true;
+    return RPBA_OK;
+  }
+  RPBA_CUDA(cudaStreamSynchronize(st));
+  if (iters) *iters = pcg_loop_steps(ctx, nullptr);
+  pcg_loop_account(ctx, nullptr);
+  return RPBA_OK;
+}
+
 rpba_status pcg_loop(Ctx *ctx, const FsaiApply *fsai, int *iters) {
   if (!fsai && ff_pcg(ctx)) {
-    if (ctx->capture && pcg_device_loop(ctx)) {
-      if (iters) *iters = 0;  // known after the replay (pinned counters)
-      return pcg_loop_device(ctx);
+    if (pcg_device_loop(ctx)) {
+      if (ctx->pcg_fused) return pcg_solve(ctx, iters);
+      if (ctx->capture) {
+        if (iters) *iters = 0;  // known after the replay (pinned counters)
+        return pcg_loop_device(ctx);
+      }
     }
     return pcg_loop_refined(ctx, iters);
   }

@@ -717,7 +717,7 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
     // solver 1 or auto's PCG in the FP32 form: float-float, for sub-blocks of
     // up to RPBA_PCG_FF_MAX_N unknowns (the step kernel's register batches)
     if (ctx->opt.precision == 1 && ctx->opt.solver == 1 && max_n <= RPBA_PCG_FF_MAX_N) {
-      ctx->pcg_ff_smem = (size_t)std::max(max_n, 1) * 2 * sizeof(float);
+      RPBA_TRY(pcg_solve_setup(ctx, max_n));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_Shi, (size_t)std::max(stot, 1LL)));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_Slo, (size_t)std::max(stot, 1LL)));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_fx, (size_t)std::max(yt, 1)));
@@ -729,11 +729,12 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_Minv32, (size_t)ctx->cd * ctx->cd * std::max(M, 1)));
       // streams on which the device-driven loop's bodies are captured (none:
       // the host-driven loop)
-      for (cudaStream_t &bs : ctx->pcg_body_stream)
-        if (cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) != cudaSuccess) {
-          cudaGetLastError();
-          bs = nullptr;
-        }
+      if (!ctx->pcg_fused)
+        for (cudaStream_t &bs : ctx->pcg_body_stream)
+          if (cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            bs = nullptr;
+          }
     }
     std::vector<int> pt(L + 1, 0);
     for (int l = 0; l < L; l++) pt[l + 1] = pt[l] + ntiles[l] * (ntiles[l] + 1) / 2;
@@ -784,8 +785,8 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
     ctx->red_blocks = (int)std::max(1LL, std::min<long long>(8LL * sms, ((long long)K + 2047) / 2048));
   }
   RPBA_TRY(alloc_n(ctx, &ctx->red, (size_t)ctx->red_blocks * 6 + 16));
-  RPBA_TRY(alloc_n(ctx, &ctx->counters, 16));
-  RPBA_CUDA(cudaMallocHost((void **)&ctx->h_pinned_counter, 16 * sizeof(int)));
+  RPBA_TRY(alloc_n(ctx, &ctx->counters, 32));
+  RPBA_CUDA(cudaMallocHost((void **)&ctx->h_pinned_counter, 32 * sizeof(int)));
   RPBA_CUDA(cudaMallocHost((void **)&ctx->h_pinned_d, 16 * sizeof(double)));
   // state: rotations from the poses, unit weights, instance copies at X
   if (M) RPBA_KERNEL(ctx, "k_pose_to_R", k_pose_to_R<<<nblk(M, 128), 128, 0, ctx->stream>>>(M, pose_d, ctx->R, ctx->t));
@@ -1418,17 +1419,7 @@ static rpba_status account(Ctx *ctx, GraphRec *g) {
     ctx->launches++;
     ctx->launch_by_name[k]++;
   }
-  if (g->pcg_loop) {  // the loop bodies ran as often as their counters say
-    long long steps = ctx->h_pinned_counter[PCG_LOOP_COUNTERS], stages = ctx->h_pinned_counter[PCG_LOOP_COUNTERS + 1];
-    for (const char *k : g->loop_inner) {
-      ctx->launches += steps;
-      ctx->launch_by_name[k] += steps;
-    }
-    for (const char *k : g->loop_outer) {
-      ctx->launches += stages;
-      ctx->launch_by_name[k] += stages;
-    }
-  }
+  if (g->pcg_loop) pcg_loop_account(ctx, g);
   if (ctx->prof_enabled)
     for (auto &ev : g->events) {
       float t = 0.f;
@@ -1439,9 +1430,9 @@ static rpba_status account(Ctx *ctx, GraphRec *g) {
 }
 
 // one lock-step LM iteration, then the host reads the running count. Direct
-// solvers, and the FP32 form's block-Jacobi PCG (its loop as conditional
-// graph nodes): one captured graph. Other PCG solvers, or a timed loop
-// kernel: a graph up to the CG start, the CG loop run from the host (it
+// solvers, and the FP32 form's block-Jacobi PCG (its loop one kernel or
+// conditional graph nodes): one captured graph. Other PCG solvers, or a timed
+// loop kernel: a graph up to the CG start, the CG loop run from the host (it
 // stops on count reads), and a graph from the back-substitution on.
 static rpba_status lm_step_exec(Ctx *ctx) {
   GraphRec *any = ctx->lm_graph ? ctx->lm_graph : ctx->lm_graph_pre;
@@ -1457,7 +1448,7 @@ static rpba_status lm_step_exec(Ctx *ctx) {
       if (ctx->lm_graph) {
         RPBA_CUDA(cudaGraphLaunch(ctx->lm_graph->exec, ctx->stream));
         RPBA_TRY(sync(ctx));
-        if (ctx->auto_solver && ctx->h_pinned_counter[PCG_LOOP_COUNTERS] > RPBA_AUTO_PCG_MAX_ITER_FP32)
+        if (ctx->auto_solver && pcg_loop_steps(ctx, nullptr) > RPBA_AUTO_PCG_MAX_ITER_FP32)
           ctx->auto_switch = true;
         return account(ctx, ctx->lm_graph);
       }

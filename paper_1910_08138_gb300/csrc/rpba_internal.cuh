@@ -326,7 +326,13 @@ struct Ctx {
   int2 *pcg_tile_map = nullptr;           // per lower tile of the running RCS: (sub-block, a << 16 | b)
   float *pcg_Minv32 = nullptr, *pcg_s32 = nullptr;
   int *pcg_act = nullptr;
-  size_t pcg_ff_smem = 0;  // the FP32 step's shared memory: r and z of the largest sub-block
+  // the loop as one kernel, k_pcg_solve: whether it is used; CTAs per cluster,
+  // whether M^-1 is in shared memory, whether the tiles stay in registers, its
+  // shared memory
+  bool pcg_fused = false, pcg_res = false;
+  int pcg_cluster = 1, pcg_minv_smem = 0;
+  size_t pcg_ff_smem = 0;  // the step kernel's shared memory: r and z of the largest sub-block
+  size_t pcg_solve_smem = 0;
   int pcg_pred = 8;        // CG iterations of the previous solve: the first convergence read
   int pcg_pred_stage[8] = {8, 8, 8, 8, 8, 8, 8, 8};  // the same per refinement stage
   // the loop as conditional graph nodes: two streams on which its bodies are
@@ -478,9 +484,9 @@ struct GraphRec {
   bool with_events = false;  // captured with per-kernel event-record nodes
   std::string prof_only;     // ... for this kernel only (empty: all)
   std::vector<const char *> kernels;
-  // the FP32-form PCG loop as conditional while nodes: the kernels of the
-  // inner (CG step) and outer (refinement stage) bodies, counted per replay
-  // from the loop's device counters
+  // holds the FP32-form PCG loop, counted per replay from its device counters:
+  // k_pcg_solve, or conditional while nodes with the kernels of the inner (CG
+  // step) and outer (refinement stage) bodies
   bool pcg_loop = false;
   std::vector<const char *> loop_inner, loop_outer;
   struct Ev {
@@ -591,7 +597,7 @@ rpba_status pcg_init(Ctx *ctx, const int *run_dev, int *fail_dev, const FsaiAppl
 // the FP32 form's block-Jacobi PCG runs as FP32 CG stages refined by
 // float-float residuals (solver 1, also when chosen by solver 4) when no
 // sub-block has more than RPBA_PCG_FF_MAX_N unknowns (256 threads x 8
-// elements in registers; r and z, 4 B each, then take at most 16 KB of shared
+// elements in registers; x, r, z and p, 4 B each, take at most 32 KB of shared
 // memory). A stage stops at RPBA_PCG_INNER_TOL of its right-hand side (or
 // sooner, where the final tolerance asks for less); at most
 // RPBA_PCG_MAX_STAGES stages per solve.
@@ -602,13 +608,17 @@ rpba_status pcg_init(Ctx *ctx, const int *run_dev, int *fail_dev, const FsaiAppl
 #define PCG_S32_STAGES 4 // the word counting the stages of the last solve
 inline bool ff_pcg(const Ctx *ctx) { return ctx->pcg_Shi != nullptr && ctx->opt.solver == 1; }
 rpba_status pcg_loop(Ctx *ctx, const FsaiApply *fsai, int *iters /* lock-step iterations run, nullable */);
-// counters of the device-driven FP32-form loop: lock-step CG steps and
-// refinement stages of the last solve (device counters[12, 14), copied to
-// h_pinned_counter[12, 14) by the captured graph)
-#define PCG_LOOP_COUNTERS 12
-// the FP32-form PCG loop runs as conditional graph nodes when the LM step is
-// captured (the context's body streams exist and no loop kernel is timed)
+// counters of the device-driven FP32-form loop at device counters[16, 25),
+// copied to h_pinned_counter[16, 25). k_pcg_solve: per refinement stage the most
+// CG steps of any sub-block (RPBA_PCG_MAX_STAGES), then the most stages; the
+// graph nodes: lock-step CG steps, stages
+#define PCG_LOOP_COUNTERS 16
+int pcg_loop_steps(const Ctx *ctx, int *stages);
+void pcg_loop_account(Ctx *ctx, const GraphRec *g);
+// the FP32-form PCG loop runs on the device (one kernel, or conditional graph
+// nodes when the LM step is captured), unless a loop kernel is being timed
 bool pcg_device_loop(const Ctx *ctx);
+rpba_status pcg_solve_setup(Ctx *ctx, int max_n);
 rpba_status pcg_out(Ctx *ctx, const int *run_dev, const int *fail_dev);
 rpba_status pcg_bj_setup(Ctx *ctx, const int *run_dev, int *fail_dev);
 rpba_status learned_setup(Ctx *ctx, const int *run_dev, int *fail_dev, FsaiApply *F);
