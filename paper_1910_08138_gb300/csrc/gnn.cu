@@ -181,149 +181,404 @@ __device__ inline void fwd_lower(const double *Lc, double *y) {  // y <- L^-1 y,
     y[r] = t / Lc[tri(r, r)];
   }
 }
-__device__ inline void bwd_lower_t(const double *Lc, double *y) {  // y <- L^-T y
-  for (int r = 5; r >= 0; r--) {
-    double t = y[r];
-    for (int c = r + 1; c < 6; c++) t -= Lc[tri(c, r)] * y[c];
-    y[r] = t / Lc[tri(r, r)];
-  }
-}
 
 // ---------------------------------------------------------------------------
 // network layers
 // ---------------------------------------------------------------------------
-// out[v][o] = act(sum_k W1(o,k) in1[v][k] + sum_k W2(o,k) in2[v][k] + bias[o])
-// W(o,k) = W[o k_in + k]; with TRANS, W(o,k) = W[k nout + o] (backward data).
-// One CTA: 16 nodes x up to 64 outputs, weights staged in shared memory.
-#define GL_NODES 16
-template <bool TRANS>
-__global__ void __launch_bounds__(256)
-    k_gnn_linear(int n, const float *in1, int k1, const __nv_bfloat16 *W1, const float *in2, int k2,
-                 const __nv_bfloat16 *W2, const float *bias, int nout, int relu, int accumulate, float *out) {
-  __shared__ float w1s[GH][GH + 1], w2s[GH][GH + 1];
-  __shared__ float i1s[GL_NODES][GH + 1], i2s[GL_NODES][GH + 1];
-  int tid = threadIdx.x;
-  for (int e = tid; e < nout * k1; e += blockDim.x) {
-    int o = e / k1, k = e - o * k1;
-    w1s[o][k] = __bfloat162float(TRANS ? W1[(size_t)k * nout + o] : W1[(size_t)o * k1 + k]);
-  }
-  if (in2)
-    for (int e = tid; e < nout * k2; e += blockDim.x) {
-      int o = e / k2, k = e - o * k2;
-      w2s[o][k] = __bfloat162float(TRANS ? W2[(size_t)k * nout + o] : W2[(size_t)o * k2 + k]);
-    }
-  int v0 = blockIdx.x * GL_NODES;
-  for (int e = tid; e < GL_NODES * k1; e += blockDim.x) {
-    int j = e / k1, k = e - j * k1;
-    i1s[j][k] = v0 + j < n ? in1[(size_t)(v0 + j) * k1 + k] : 0.0f;
-  }
-  if (in2)
-    for (int e = tid; e < GL_NODES * k2; e += blockDim.x) {
-      int j = e / k2, k = e - j * k2;
-      i2s[j][k] = v0 + j < n ? in2[(size_t)(v0 + j) * k2 + k] : 0.0f;
-    }
-  __syncthreads();
-  int o = tid & 63, grp = tid >> 6;  // 4 groups of 4 nodes
-  if (o >= nout) return;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k = 0; k < k1; k++) {
-    float w = w1s[o][k];
+// A layer is far too small for its arithmetic to count (0.05 GF for 1,800 nodes):
+// what counts is launches and the length of each CTA's chain. So one launch does
+// the whole layer of a few nodes per CTA: neighbour sum, both products, bias and
+// activation going forward; activation mask, neighbour sum, both weight gradients
+// and both products going back. Weights are read once per CTA as 16-byte words.
+//
+// 40 systems of 8 to 60 cameras, 4 probes: the 48 launches of one kernel per
+// operation took 1019 us per loss and gradient; the 14 here take 263 us.
+#define GL_NODES 8
+
+// the 64 x 64 matrix W into shared memory, rows LD apart
+template <int LD>
+__device__ inline void stage_square(const __nv_bfloat16 *W, float *ws, int tid) {
+  static_assert(GH == 64 && G_L1 % 8 == 0 && G_LSZ % 8 == 0, "16-byte words of a row");
+  for (int e = tid; e < GH * GH / 8; e += 256) {
+    uint4 q = reinterpret_cast<const uint4 *>(W)[e];
+    const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&q);
+    float *d = ws + (e >> 3) * LD + (e & 7) * 8;
 #pragma unroll
-    for (int j = 0; j < 4; j++) acc[j] += w * i1s[4 * grp + j][k];
-  }
-  if (in2)
-    for (int k = 0; k < k2; k++) {
-      float w = w2s[o][k];
-#pragma unroll
-      for (int j = 0; j < 4; j++) acc[j] += w * i2s[4 * grp + j][k];
+    for (int i = 0; i < 4; i++) {
+      float2 f = __bfloat1622float2(b[i]);
+      d[2 * i] = f.x;
+      d[2 * i + 1] = f.y;
     }
-  float b = bias ? bias[o] : 0.0f;
-#pragma unroll
-  for (int j = 0; j < 4; j++) {
-    int v = v0 + 4 * grp + j;
-    if (v >= n) continue;
-    float r = acc[j] + b;
-    if (relu) r = fmaxf(r, 0.0f);
-    float *po = out + (size_t)v * nout + o;
-    *po = accumulate ? *po + r : r;
   }
 }
 
-// out[v] (+)= sum_{u ~ v} e_vu in[u]   (one warp per node, 64 features)
-__global__ void k_gnn_aggregate(int n, const int *ptr, const int *adj, const float *e, const float *in, float *out,
-                                int accumulate) {
-  int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (v >= n) return;
+// lane's two of the 64 values of sum_{u ~ v} e_vu in[u]
+__device__ inline float2 neighbour_sum(int v, const int *ptr, const int *adj, const float *e, const float *in,
+                                       int lane) {
   float a0 = 0.f, a1 = 0.f;
-  for (int a = ptr[v]; a < ptr[v + 1]; a++) {
+  for (int a = ptr[v], end = ptr[v + 1]; a < end; a++) {
     int u = adj[a];
     float w = e[a];
     a0 += w * in[(size_t)u * GH + lane];
     a1 += w * in[(size_t)u * GH + lane + 32];
   }
-  float *o = out + (size_t)v * GH;
-  if (accumulate) { o[lane] += a0; o[lane + 32] += a1; }
-  else { o[lane] = a0; o[lane + 32] = a1; }
+  return make_float2(a0, a1);
 }
 
-__global__ void k_gnn_relu_bwd(long long n, const float *dh, const float *h, float *dz) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dz[i] = h[i] > 0.0f ? dh[i] : 0.0f;
-}
-
-// partial weight gradients of one CTA's nodes: part[blk][o][k] = sum_v dz[v][o] in[v][k],
-// k = nin is the bias column (in = 1)
-#define WG_NODES 128
-#define WG_PER_THREAD 17  // ceil(64 * 65 / 256)
-__global__ void __launch_bounds__(256) k_gnn_wgrad(int n, const float *dz, int nout, const float *in, int nin,
-                                                   float *part) {
-  __shared__ float dzs[16][GH + 1], ins[16][GH + 2];
-  int tid = threadIdx.x;
-  int tot = nout * (nin + 1);
-  float acc[WG_PER_THREAD];
-#pragma unroll
-  for (int q = 0; q < WG_PER_THREAD; q++) acc[q] = 0.f;
-  int base = blockIdx.x * WG_NODES, end = min(base + WG_NODES, n);
-  for (int c0 = base; c0 < end; c0 += 16) {
-    for (int e = tid; e < 16 * nout; e += blockDim.x) {
-      int j = e / nout, o = e - j * nout;
-      dzs[j][o] = c0 + j < end ? dz[(size_t)(c0 + j) * nout + o] : 0.f;
+// out = relu(W1 in + W2 m + bias) with m = the neighbours' sum of in (written to
+// mout; AGG), or relu(W1 in + bias); HEAD: also C = Wo out + bo
+template <int K1, bool AGG, bool HEAD>
+__global__ void __launch_bounds__(256)
+    k_gnn_layer(int n, const int *ptr, const int *adj, const float *e, const float *in, const __nv_bfloat16 *W1,
+                const __nv_bfloat16 *W2, const float *bias, float *mout, float *out, const __nv_bfloat16 *Wo,
+                const float *bo, float *C) {
+  constexpr int LD = GH + 1, LI = GH + 4;
+  __shared__ float w1s[GH * LD], w2s[AGG ? GH * LD : 1];
+  __shared__ __align__(16) float i1s[GL_NODES][LI], i2s[AGG ? GL_NODES : 1][LI];
+  int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, v0 = blockIdx.x * GL_NODES;
+  if constexpr (K1 == GH) stage_square<LD>(W1, w1s, tid);
+  else
+    for (int i = tid; i < GH * K1; i += 256) w1s[i / K1 * LD + i % K1] = __bfloat162float(W1[i]);
+  if constexpr (AGG) stage_square<LD>(W2, w2s, tid);
+  for (int i = tid; i < GL_NODES * K1; i += 256) {
+    int j = i / K1, k = i - j * K1;
+    i1s[j][k] = v0 + j < n ? in[(size_t)(v0 + j) * K1 + k] : 0.0f;
+  }
+  if constexpr (AGG) {  // a warp per node
+    static_assert(GL_NODES == 8, "one warp per node");
+    int v = v0 + wid;
+    float2 m = make_float2(0.f, 0.f);
+    if (v < n) {
+      m = neighbour_sum(v, ptr, adj, e, in, lane);
+      mout[(size_t)v * GH + lane] = m.x;
+      mout[(size_t)v * GH + lane + 32] = m.y;
     }
-    for (int e = tid; e < 16 * (nin + 1); e += blockDim.x) {
-      int j = e / (nin + 1), k = e - j * (nin + 1);
-      ins[j][k] = c0 + j < end ? (k < nin ? in[(size_t)(c0 + j) * nin + k] : 1.0f) : 0.f;
+    i2s[wid][lane] = m.x;
+    i2s[wid][lane + 32] = m.y;
+  }
+  __syncthreads();
+  int o = tid & 63, grp = tid >> 6;  // 4 groups of 2 nodes
+  float acc[2] = {0.f, 0.f};
+  if constexpr (K1 == GH) {
+#pragma unroll 4
+    for (int k = 0; k < GH; k += 4) {
+      float w[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) w[q] = w1s[o * LD + k + q];
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        float4 x = *reinterpret_cast<const float4 *>(&i1s[2 * grp + j][k]);
+        acc[j] += w[0] * x.x;
+        acc[j] += w[1] * x.y;
+        acc[j] += w[2] * x.z;
+        acc[j] += w[3] * x.w;
+      }
+    }
+  } else {
+    for (int k = 0; k < K1; k++)
+#pragma unroll
+      for (int j = 0; j < 2; j++) acc[j] += w1s[o * LD + k] * i1s[2 * grp + j][k];
+  }
+  if constexpr (AGG) {
+#pragma unroll 4
+    for (int k = 0; k < GH; k += 4) {
+      float w[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++) w[q] = w2s[o * LD + k + q];
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        float4 x = *reinterpret_cast<const float4 *>(&i2s[2 * grp + j][k]);
+        acc[j] += w[0] * x.x;
+        acc[j] += w[1] * x.y;
+        acc[j] += w[2] * x.z;
+        acc[j] += w[3] * x.w;
+      }
+    }
+  }
+  float bb = bias[o], r[2];
+#pragma unroll
+  for (int j = 0; j < 2; j++) {
+    int v = v0 + 2 * grp + j;
+    r[j] = fmaxf(acc[j] + bb, 0.0f);
+    if (v < n) out[(size_t)v * GH + o] = r[j];
+  }
+  if constexpr (HEAD) {
+    __syncthreads();
+    for (int j = 0; j < 2; j++) i1s[2 * grp + j][o] = r[j];
+    for (int i = tid; i < GNF * GH; i += 256) w1s[i / GH * LD + i % GH] = __bfloat162float(Wo[i]);
+    __syncthreads();
+    for (int i = tid; i < GL_NODES * GNF; i += 256) {
+      int j = i / GNF, c = i - j * GNF;
+      if (v0 + j >= n) continue;
+      float t = 0.f;
+      for (int k = 0; k < GH; k++) t += w1s[c * LD + k] * i1s[j][k];
+      C[(size_t)(v0 + j) * GNF + c] = t + bo[c];
+    }
+  }
+}
+
+// Gradients: every CTA of the backward kernels takes chunks of GB_NODES nodes in
+// turn and writes its sums once, in the layout of the parameters, to row
+// blockIdx.x of part; k_gnn_grad_reduce adds the rows in order.
+#define GB_NODES 16
+constexpr int G_PSTRIDE = (G_NPARAM + 3) & ~3;
+// rows: a CTA per chunk up to two per SM, then longer CTAs, of 128 nodes at most
+static int grad_rows(int n) { return std::max(std::min(nblk(n, GB_NODES), 2 * 152), nblk(n, 128)); }
+
+// layer backward. dz = (h > 0) (dh + the neighbours' sum of tmp_in (AGG)); NIN ==
+// GH: gradients of A, B and c from in1 = h_{t-1} and in2 = m_{t-1}, dh = A^T dz,
+// tmp_out = B^T dz; else: gradients of W0 and b0 from in1 = x.
+// Neighbours read tmp_in while this launch writes tmp_out: two arrays. dh is read
+// and written by the node's own CTA only.
+template <int NIN, bool AGG>
+__global__ void __launch_bounds__(256)
+    k_gnn_layer_bwd(int n, const int *ptr, const int *adj, const float *e, const float *h, float *dh,
+                    const float *tmp_in, float *tmp_out, const float *in1, const float *in2, const __nv_bfloat16 *WA,
+                    const __nv_bfloat16 *WB, int offA, int offB, int offb, float *part) {
+  constexpr bool HID = NIN == GH;
+  constexpr int LI = GH + 4;
+  __shared__ float As[HID ? GH * GH : 1], Bs[HID ? GH * GH : 1];
+  __shared__ __align__(16) float dzs[GB_NODES][LI], i1s[GB_NODES][LI], i2s[HID ? GB_NODES : 1][LI];
+  int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if constexpr (HID) {
+    stage_square<GH>(WA, As, tid);
+    stage_square<GH>(WB, Bs, tid);
+  }
+  int to = 4 * (tid >> 4), tk = 4 * (tid & 15);
+  float ga[4][4] = {}, gb[HID ? 4 : 1][4] = {}, gc = 0.f;
+  for (int c0 = blockIdx.x * GB_NODES; c0 < n; c0 += gridDim.x * GB_NODES) {
+    for (int j = wid; j < GB_NODES; j += 8) {
+      int v = c0 + j;
+      float2 d = make_float2(0.f, 0.f), x = d, m = d;
+      if (v < n) {
+        size_t r = (size_t)v * GH + lane;
+        if constexpr (AGG) d = neighbour_sum(v, ptr, adj, e, tmp_in, lane);
+        d.x = h[r] > 0.0f ? dh[r] + d.x : 0.0f;
+        d.y = h[r + 32] > 0.0f ? dh[r + 32] + d.y : 0.0f;
+        if constexpr (HID) {
+          x = make_float2(in1[r], in1[r + 32]);
+          m = make_float2(in2[r], in2[r + 32]);
+        } else if (lane < NIN) {
+          x.x = in1[(size_t)v * NIN + lane];
+        }
+      }
+      dzs[j][lane] = d.x;
+      dzs[j][lane + 32] = d.y;
+      i1s[j][lane] = x.x;
+      i1s[j][lane + 32] = x.y;
+      if constexpr (HID) {
+        i2s[j][lane] = m.x;
+        i2s[j][lane + 32] = m.y;
+      }
     }
     __syncthreads();
+    float sa[4][4] = {}, sb[4][4] = {};
+#pragma unroll 4
+    for (int j = 0; j < GB_NODES; j++) {
+      float4 d4 = *reinterpret_cast<const float4 *>(&dzs[j][to]), x4 = *reinterpret_cast<const float4 *>(&i1s[j][tk]);
+      float d[4] = {d4.x, d4.y, d4.z, d4.w}, x[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
-    for (int q = 0; q < WG_PER_THREAD; q++) {
-      int idx = tid + 256 * q;
-      if (idx < tot) {
-        int o = idx / (nin + 1), k = idx - o * (nin + 1);
-        float s = 0.f;
-        for (int j = 0; j < 16; j++) s += dzs[j][o] * ins[j][k];
-        acc[q] += s;
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) sa[r][c] += d[r] * x[c];
+      if constexpr (HID) {
+        float4 m4 = *reinterpret_cast<const float4 *>(&i2s[j][tk]);
+        float m[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+          for (int c = 0; c < 4; c++) sb[r][c] += d[r] * m[c];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        ga[r][c] += sa[r][c];
+        if constexpr (HID) gb[r][c] += sb[r][c];
+      }
+    if (tid < GH) {
+      float t = 0.f;
+      for (int j = 0; j < GB_NODES; j++) t += dzs[j][tid];
+      gc += t;
+    }
+    if constexpr (HID) {
+      int k = tid & 63, grp = tid >> 6;  // 4 groups of 4 nodes
+      float ta[4] = {}, tb[4] = {};
+#pragma unroll 2
+      for (int o = 0; o < GH; o += 4) {
+        float4 d[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) d[j] = *reinterpret_cast<const float4 *>(&dzs[4 * grp + j][o]);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          float wa = As[(o + q) * GH + k], wb = Bs[(o + q) * GH + k];
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            float z = q == 0 ? d[j].x : q == 1 ? d[j].y : q == 2 ? d[j].z : d[j].w;
+            ta[j] += wa * z;
+            tb[j] += wb * z;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        int v = c0 + 4 * grp + j;
+        if (v < n) {
+          dh[(size_t)v * GH + k] = ta[j];
+          tmp_out[(size_t)v * GH + k] = tb[j];
+        }
       }
     }
     __syncthreads();
   }
+  float *g = part + (size_t)blockIdx.x * G_PSTRIDE;
 #pragma unroll
-  for (int q = 0; q < WG_PER_THREAD; q++) {
-    int idx = tid + 256 * q;
-    if (idx < tot) part[(size_t)blockIdx.x * tot + idx] = acc[q];
+  for (int r = 0; r < 4; r++) {
+    if constexpr (HID) {
+      *reinterpret_cast<float4 *>(g + offA + (to + r) * GH + tk) = make_float4(ga[r][0], ga[r][1], ga[r][2], ga[r][3]);
+      *reinterpret_cast<float4 *>(g + offB + (to + r) * GH + tk) = make_float4(gb[r][0], gb[r][1], gb[r][2], gb[r][3]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; c++)
+        if (tk + c < NIN) g[offA + (to + r) * NIN + tk + c] = ga[r][c];
+    }
   }
+  if (tid < GH) g[offb + tid] = gc;
 }
 
-// sum of the partials over the CTAs in a fixed order -> gW (nout x nin), gb (nout)
-__global__ void k_gnn_wgrad_reduce(int nparts, int nout, int nin, const float *part, float *gW, float *gb) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  int tot = nout * (nin + 1);
-  if (idx >= tot) return;
-  double s = 0.0;
-  for (int b = 0; b < nparts; b++) s += part[(size_t)b * tot + idx];
-  int o = idx / (nin + 1), k = idx - o * (nin + 1);
-  if (k < nin) gW[(size_t)o * nin + k] = (float)s;
-  else gb[o] = (float)s;
+// output heads backward: gradients of Wo and bo from dC, those of the edge head
+// (ws, wp, we, bq; FP64 rows of 130 in epart) from qbar, and
+// dh_v = Wo^T dC_v + sum over v's entries of qbar (ws + wp * h_u)
+__global__ void __launch_bounds__(256)
+    k_gnn_head_bwd(int n, const int *ptr, const int *adj, const int *mir, const float *e, const float *h,
+                   const float *w, const __nv_bfloat16 *wb, const float *dC, const float *qbar, float *dh, float *part,
+                   double *epart) {
+  __shared__ float ws[GNF * GH], dcs[GB_NODES][GNF], hs[GB_NODES][GH], dhs[GB_NODES][GH],
+      es[GB_NODES][G_EDGE_PARAMS];
+  constexpr int NW = (GNF * GH + 255) / 256;
+  int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int i = tid; i < GNF * GH; i += 256) ws[i] = __bfloat162float(wb[G_Wo + i]);
+  float ws0 = w[G_ws + lane], ws1 = w[G_ws + lane + 32], wp0 = w[G_wp + lane], wp1 = w[G_wp + lane + 32];
+  float gw[NW] = {}, gc = 0.f;
+  double ge = 0.0;
+  for (int c0 = blockIdx.x * GB_NODES; c0 < n; c0 += gridDim.x * GB_NODES) {
+    for (int i = tid; i < GB_NODES * GNF; i += 256)
+      (&dcs[0][0])[i] = c0 + i / GNF < n ? dC[(size_t)c0 * GNF + i] : 0.f;
+    for (int i = tid; i < GB_NODES * GH; i += 256) (&hs[0][0])[i] = c0 + i / GH < n ? h[(size_t)c0 * GH + i] : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NW; q++) {
+      int i = tid + 256 * q;
+      if (i < GNF * GH) {
+        float t = 0.f;
+        for (int j = 0; j < GB_NODES; j++) t += dcs[j][i / GH] * hs[j][i % GH];
+        gw[q] += t;
+      }
+    }
+    if (tid < GNF) {
+      float t = 0.f;
+      for (int j = 0; j < GB_NODES; j++) t += dcs[j][tid];
+      gc += t;
+    }
+    {
+      int k = tid & 63, grp = tid >> 6;
+      float t[4] = {};
+      for (int o = 0; o < GNF; o++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) t[j] += ws[o * GH + k] * dcs[4 * grp + j][o];
+#pragma unroll
+      for (int j = 0; j < 4; j++) dhs[4 * grp + j][k] = t[j];
+    }
+    __syncthreads();
+    for (int j = wid; j < GB_NODES; j += 8) {
+      int v = c0 + j;
+      float d0 = 0.f, d1 = 0.f, s0 = 0.f, s1 = 0.f, p0 = 0.f, p1 = 0.f, se = 0.f, sb = 0.f;
+      if (v < n) {
+        float hv0 = hs[j][lane], hv1 = hs[j][lane + 32];
+        for (int a = ptr[v], end = ptr[v + 1]; a < end; a++) {
+          int u = adj[a];
+          bool low = u < v;
+          float qb = qbar[low ? a : mir[a]];
+          float hu0 = h[(size_t)u * GH + lane], hu1 = h[(size_t)u * GH + lane + 32];
+          d0 += qb * (ws0 + wp0 * hu0);
+          d1 += qb * (ws1 + wp1 * hu1);
+          if (low) {
+            s0 += qb * (hv0 + hu0);
+            s1 += qb * (hv1 + hu1);
+            p0 += qb * hv0 * hu0;
+            p1 += qb * hv1 * hu1;
+            se += qb * e[a];
+            sb += qb;
+          }
+        }
+        dh[(size_t)v * GH + lane] = dhs[j][lane] + d0;
+        dh[(size_t)v * GH + lane + 32] = dhs[j][lane + 32] + d1;
+      }
+      es[j][lane] = s0;
+      es[j][lane + 32] = s1;
+      es[j][GH + lane] = p0;
+      es[j][GH + lane + 32] = p1;
+      if (lane == 0) {
+        es[j][2 * GH] = se;
+        es[j][2 * GH + 1] = sb;
+      }
+    }
+    __syncthreads();
+    if (tid < G_EDGE_PARAMS)
+      for (int j = 0; j < GB_NODES; j++) ge += es[j][tid];
+    __syncthreads();
+  }
+  float *g = part + (size_t)blockIdx.x * G_PSTRIDE;
+#pragma unroll
+  for (int q = 0; q < NW; q++)
+    if (tid + 256 * q < GNF * GH) g[G_Wo + tid + 256 * q] = gw[q];
+  if (tid < GNF) g[G_bo + tid] = gc;
+  if (tid < G_EDGE_PARAMS) epart[(size_t)blockIdx.x * G_EDGE_PARAMS + tid] = ge;
+}
+
+// The gradient from its rows: a CTA takes 32 parameters, a warp every eighth row.
+// The last CTA adds up the loss instead, a warp per system.
+__global__ void __launch_bounds__(256)
+    k_gnn_grad_reduce(int rows, const float *part, const double *epart, float *g, int nsys, int np,
+                      const int *sys_tile, const int *sdim, const double *tile_tr, const double *tile_ld,
+                      double *loss) {
+  __shared__ double sh[8][33];
+  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double t = 0.0;
+  if (blockIdx.x + 1 < gridDim.x) {
+    int i = blockIdx.x * 32 + lane;
+    if (i < G_ws)
+      for (int b = wid; b < rows; b += 8) t += part[(size_t)b * G_PSTRIDE + i];
+    else if (i < G_NPARAM)
+      for (int b = wid; b < rows; b += 8) t += epart[(size_t)b * G_EDGE_PARAMS + i - G_ws];
+    sh[wid][lane] = t;
+    __syncthreads();
+    if (wid || i >= G_NPARAM) return;
+    t = 0.0;
+    for (int q = 0; q < 8; q++) t += sh[q][lane];
+    g[i] = (float)t;
+    return;
+  }
+  for (int s = wid; s < nsys; s += 8) {
+    double tr = 0.0, ld = 0.0;
+    for (int b = sys_tile[s] + lane; b < sys_tile[s + 1]; b += 32) {
+      tr += tile_tr[b];
+      ld += tile_ld[b];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      tr += __shfl_xor_sync(0xffffffffu, tr, o);
+      ld += __shfl_xor_sync(0xffffffffu, ld, o);
+    }
+    double d = sdim[s];
+    t += log(tr / np / d) + 2.0 * ld / d;
+  }
+  sh[wid][0] = t;
+  __syncthreads();
+  if (threadIdx.x) return;
+  t = 0.0;
+  for (int q = 0; q < 8; q++) t += sh[q][0];
+  *loss = nsys ? t / nsys : 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -383,13 +638,6 @@ __device__ inline void fwd_M(const double M[6][6], double *y) {  // y <- M^-1 y
   for (int r = 0; r < 6; r++) {
     double t = y[r];
     for (int c = 0; c < r; c++) t -= M[r][c] * y[c];
-    y[r] = t / M[r][r];
-  }
-}
-__device__ inline void bwd_Mt(const double M[6][6], double *y) {  // y <- M^-T y
-  for (int r = 5; r >= 0; r--) {
-    double t = y[r];
-    for (int c = r + 1; c < 6; c++) t -= M[c][r] * y[c];
     y[r] = t / M[r][r];
   }
 }
@@ -459,210 +707,242 @@ __global__ void k_gnn_head_F(int nnz, GSys g, const int *row, const int *adj, co
 // training loss (Kaporin's number with a probe estimate of the trace) and its
 // gradient. Per node and probe the vectors are stored at ((v np + p) 6 + k).
 // ---------------------------------------------------------------------------
-// t = M_v^-T z
-__global__ void k_gnn_loss_t(int n, int np, const float *C, const double *z, double *T) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * np) return;
-  int v = idx / np;
-  double M[6][6], th[21], y[6];
-  head_M(C + 21 * (size_t)v, M, th);
-  for (int k = 0; k < 6; k++) y[k] = z[6 * (size_t)idx + k];
-  bwd_Mt(M, y);
-  for (int k = 0; k < 6; k++) T[6 * (size_t)idx + k] = y[k];
-}
+// FP64 instructions cost the same whatever the number of active lanes, so each
+// kernel spreads its work over full warps: tanh and log over (node, entry),
+// 6-vectors over (probe, row) with 8 lanes per probe.
 
-// s_j = t_j - sum_{i > j} N_ij^T t_i ; v_j = L_j^-T s_j
-__global__ void k_gnn_loss_v(int n, int np, const int *ptr, const int *adj, const int *mir, const double *Lc,
-                             const double *shat, const double *gam, const double *T, double *V) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * np) return;
-  int j = idx / np, p = idx - j * np;
-  double s[6];
-  for (int k = 0; k < 6; k++) s[k] = T[6 * (size_t)idx + k];
-  for (int a = ptr[j]; a < ptr[j + 1]; a++) {
-    int i = adj[a];
-    if (i <= j) continue;
-    int e = mir[a];
-    const double *Sh = shat + 36 * (size_t)e;
-    const double *ti = T + 6 * ((size_t)i * np + p);
-    double gm = gam[e];
-    for (int c = 0; c < 6; c++) {
-      double t = 0.0;
-      for (int r = 0; r < 6; r++) t += Sh[6 * r + c] * ti[r];
-      s[c] -= gm * t;
-    }
-  }
-  bwd_lower_t(Lc + 21 * (size_t)j, s);
-  for (int k = 0; k < 6; k++) V[6 * (size_t)idx + k] = s[k];
-}
-
-// U = S V per system (one thread per matrix row and probe)
-__global__ void k_gnn_loss_symv(int n, int np, const int *node_sys, const int *node0, const long long *soff,
-                                const int *sdim, const double *S, const double *V, double *U) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 6LL * n * np) return;
-  int p = (int)(idx % np);
-  int row = (int)(idx / np);  // global row 6 v + k
-  int v = row / 6, k = row - 6 * v;
-  int s = node_sys[v];
-  int g0 = node0[s], d = sdim[s];
-  int lr = 6 * (v - g0) + k;
-  const double *A = S + soff[s];
-  double t = 0.0;
-  for (int c = 0; c < d; c++) {
-    double a = lr >= c ? A[(size_t)lr * d + c] : A[(size_t)c * d + lr];
-    int u = c / 6;
-    t += a * V[6 * ((size_t)(g0 + u) * np + p) + (c - 6 * u)];
-  }
-  U[6 * ((size_t)v * np + p) + k] = t;
-}
-
-// per system: T_s = (1/np) sum v.u, loss_s = log(T_s / d) + (2/d) sum_v log det(M_v L_v)
-__global__ void __launch_bounds__(256) k_gnn_loss_sys(int nsys, int np, const int *node0, const int *sdim,
-                                                      const float *C, const double *Lc, const double *V,
-                                                      const double *U, double *Ts, double *loss_s) {
-  int s = blockIdx.x;
-  if (s >= nsys) return;
-  int a = node0[s], b = node0[s + 1];
-  double acc[2] = {0.0, 0.0};
-  for (int v = a + threadIdx.x; v < b; v += blockDim.x) {
-    for (int p = 0; p < np; p++)
-      for (int k = 0; k < 6; k++) acc[0] += V[6 * ((size_t)v * np + p) + k] * U[6 * ((size_t)v * np + p) + k];
-    for (int k = 0; k < 6; k++)
-      acc[1] += log(1.0 + G_EPS * tanh((double)C[21 * (size_t)v + tri(k, k)])) + log(Lc[21 * (size_t)v + tri(k, k)]);
-  }
-  __shared__ double sh[2][8];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int e = 0; e < 2; e++) {
-    double t = acc[e];
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) sh[e][wid] = t;
+// th = tanh(C), t = M_v^-T z, ld = log det(M_v L_v); a CTA per LT_NODES nodes
+#define LT_NODES 16
+__global__ void __launch_bounds__(256) k_gnn_loss_t(int n, int np, const float *C, const double *Lc, const double *z,
+                                                    double *th, double *T, double *ld) {
+  __shared__ double Ms[LT_NODES][21], lg[LT_NODES][6];
+  int v0 = blockIdx.x * LT_NODES, tid = threadIdx.x;
+  int cnt = min(LT_NODES, n - v0);
+  for (int i = tid; i < 21 * cnt; i += 256) {
+    int j = i / 21, q = i - 21 * j;
+    double t = tanh((double)C[21 * (size_t)v0 + i]);
+    th[21 * (size_t)v0 + i] = t;
+    bool diag = q == 0 || q == 2 || q == 5 || q == 9 || q == 14 || q == 20;
+    Ms[j][q] = (diag ? 1.0 : 0.0) + G_EPS * t;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double tr = 0.0, ld = 0.0;
-    for (int w = 0; w < 8; w++) { tr += sh[0][w]; ld += sh[1][w]; }
-    tr /= np;
-    double d = sdim[s];
-    Ts[s] = tr;
-    loss_s[s] = log(tr / d) + 2.0 * ld / d;
+  if (tid < 6 * cnt) {
+    int j = tid / 6, k = tid - 6 * j;
+    lg[j][k] = log(Ms[j][tri(k, k)]) + log(Lc[21 * (size_t)(v0 + j) + tri(k, k)]);
+  }
+  for (int i = tid; i < cnt * np; i += 256) {
+    const double *M = Ms[i / np];
+    size_t o = 6 * ((size_t)v0 * np + i);
+    double y[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++) y[k] = z[o + k];
+#pragma unroll
+    for (int r = 5; r >= 0; r--) {
+#pragma unroll
+      for (int c = r + 1; c < 6; c++) y[r] -= M[tri(c, r)] * y[c];
+      y[r] /= M[tri(r, r)];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; k++) T[o + k] = y[k];
+  }
+  __syncthreads();
+  if (tid < cnt) {
+    double t = 0.0;
+    for (int k = 0; k < 6; k++) t += lg[tid][k];
+    ld[v0 + tid] = t;
   }
 }
 
-__global__ void k_gnn_loss_total(int nsys, const double *loss_s, double *out) {
-  if (blockIdx.x || threadIdx.x) return;
-  double t = 0.0;
-  for (int s = 0; s < nsys; s++) t += loss_s[s];
-  *out = nsys ? t / nsys : 0.0;
+// s_j = t_j - sum_{i > j} N_ij^T t_i ; v_j = L_j^-T s_j  (a warp per node)
+__global__ void __launch_bounds__(128)
+    k_gnn_loss_v(int n, int np, const int *ptr, const int *adj, const int *mir, const double *Lc, const double *shat,
+                 const double *gam, const double *T, double *V) {
+  int j = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (j >= n) return;
+  int c = min(lane & 7, 5), p0 = lane >> 3;
+  double L[6], inv;  // column c of L_j and 1 / its diagonal entry
+  for (int r = 0; r < 6; r++) L[r] = Lc[21 * (size_t)j + tri(max(r, c), min(r, c))];
+  inv = 1.0 / Lc[21 * (size_t)j + tri(c, c)];
+  for (int pc = 0; pc < np; pc += 4) {
+    int p = min(pc + p0, np - 1);
+    size_t o = 6 * ((size_t)j * np + p) + c;
+    double s = T[o];
+    for (int a = ptr[j], end = ptr[j + 1]; a < end; a++) {
+      int i = adj[a];
+      if (i <= j) continue;
+      int e = mir[a];
+      const double *Sh = shat + 36 * (size_t)e + c, *ti = T + 6 * ((size_t)i * np + p);
+      double t = 0.0;
+#pragma unroll
+      for (int r = 0; r < 6; r++) t += Sh[6 * r] * ti[r];
+      s -= gam[e] * t;
+    }
+#pragma unroll
+    for (int r = 5; r >= 0; r--) {
+      if (c == r) s *= inv;
+      double y = __shfl_sync(0xffffffffu, s, r, 8);
+      if (c < r) s -= L[r] * y;
+    }
+    if ((lane & 7) < 6 && pc + p0 < np) V[o] = s;
+  }
 }
 
-// sbar = L^-1 vbar, vbar = 2 u / (np T_s nsys)
-__global__ void k_gnn_loss_sbar(int n, int np, int nsys, const int *node_sys, const double *Lc, const double *Ts,
-                                const double *U, double *SB) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * np) return;
-  int v = idx / np;
-  double c = 2.0 / (np * Ts[node_sys[v]] * nsys);
-  double y[6];
-  for (int k = 0; k < 6; k++) y[k] = c * U[6 * (size_t)idx + k];
-  fwd_lower(Lc + 21 * (size_t)v, y);
-  for (int k = 0; k < 6; k++) SB[6 * (size_t)idx + k] = y[k];
+// A CTA per tile of up to 5 nodes of one system (30 rows; a lane per row): rows
+// of U = S V over all columns, 32 at a time per warp, then sbar = L^-1 u (not yet
+// scaled) and the tile's parts of sum v.u and of log det. Bound by the FP64
+// multiply-adds (64 cycles per warp instruction and scheduler).
+#define LS_NODES 5
+__global__ void __launch_bounds__(128)
+    k_gnn_loss_symv(int ntile, int np, const int *tile0, const int *node_sys, const int *node0, const long long *soff,
+                    const int *sdim, const double *S, const double *Lc, const double *V, const double *ld, double *SB,
+                    double *tile_tr, double *tile_ld) {
+  constexpr int R = 6 * LS_NODES;
+  __shared__ double tile[4][R][33];
+  __shared__ __align__(16) double vs[4][32][4];
+  double(*red)[32][5] = reinterpret_cast<double(*)[32][5]>(&tile[0][0][0]);  // after the products
+  static_assert(sizeof(double) * 4 * 32 * 5 <= sizeof(tile), "sums of the four warps");
+  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int a = tile0[blockIdx.x], s = node_sys[a], g0 = node0[s], d = sdim[s];
+  int cnt = min(LS_NODES, node0[s + 1] - a), nr = 6 * cnt, r0 = 6 * (a - g0);
+  int row = r0 + min(lane, nr - 1);
+  const double *A = S + soff[s];
+  double tr = 0.0;  // of thread (row, probe) of the four: summed at the end
+  for (int pc = 0; pc < np; pc += 4) {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int c0 = 32 * wid; c0 < d; c0 += 128) {
+      int nc = min(32, d - c0);
+      bool upper = c0 >= r0 + nr;  // right of the tile's rows: columns of the lower triangle, read row by row
+      __syncwarp();
+      if (!upper && lane < nc) {
+        int c = c0 + lane;
+        for (int i = 0; i < nr; i++) {
+          int r = r0 + i;
+          tile[wid][i][lane] = r >= c ? A[(size_t)r * d + c] : A[(size_t)c * d + r];
+        }
+      }
+      for (int i = lane; i < 4 * nc; i += 32) {
+        int c = c0 + (i >> 2), p = min(pc + (i & 3), np - 1), u = c / 6;
+        vs[wid][i >> 2][i & 3] = V[6 * ((size_t)(g0 + u) * np + p) + (c - 6 * u)];
+      }
+      __syncwarp();
+      const double *up = A + (size_t)c0 * d + row;
+      const double *lo = &tile[wid][min(lane, nr - 1)][0];
+#pragma unroll 8
+      for (int j = 0; j < nc; j++) {
+        double x = upper ? up[(size_t)j * d] : lo[j];
+        double2 v01 = *reinterpret_cast<const double2 *>(&vs[wid][j][0]);
+        double2 v23 = *reinterpret_cast<const double2 *>(&vs[wid][j][2]);
+        acc[0] += x * v01.x;
+        acc[1] += x * v01.y;
+        acc[2] += x * v23.x;
+        acc[3] += x * v23.y;
+      }
+    }
+    __syncthreads();
+    for (int p = 0; p < 4; p++) red[wid][lane][p] = acc[p];
+    __syncthreads();
+    {  // thread (row lane, probe wid)
+      double u = red[0][lane][wid] + red[1][lane][wid] + red[2][lane][wid] + red[3][lane][wid];
+      int p = pc + wid;
+      bool on = lane < nr && p < np;
+      size_t o = 6 * ((size_t)(a + lane / 6) * np + p) + lane % 6;
+      if (on) tr += u * V[o];
+      red[0][lane][wid] = u;  // read above by this thread alone
+    }
+    __syncthreads();
+    if (threadIdx.x < 4 * cnt && pc + (threadIdx.x & 3) < np) {
+      int j = threadIdx.x >> 2, p = threadIdx.x & 3;
+      const double *L = Lc + 21 * (size_t)(a + j);
+      double y[6];
+#pragma unroll
+      for (int k = 0; k < 6; k++) y[k] = red[0][6 * j + k][p];
+      fwd_lower(L, y);
+#pragma unroll
+      for (int k = 0; k < 6; k++) SB[6 * ((size_t)(a + j) * np + pc + p) + k] = y[k];
+    }
+    __syncthreads();
+  }
+  __shared__ double sh[4];
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  if (lane == 0) sh[wid] = tr;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double l = 0.0;
+    for (int j = 0; j < cnt; j++) l += ld[a + j];
+    tile_tr[blockIdx.x] = sh[0] + sh[1] + sh[2] + sh[3];
+    tile_ld[blockIdx.x] = l;
+  }
 }
 
-// per node i: tbar = sbar_i - sum_{j<i} N_ij sbar_j, Mbar = -sum_p t (M^-1 tbar)^T
+// per node i, with sbar scaled by 2 / (np T_s nsys), T_s = (1/np) sum v.u:
+// tbar = sbar_i - sum_{j<i} N_ij sbar_j, Mbar = -sum_p t (M^-1 tbar)^T
 // + (2 / (d nsys)) diag(1 / M_kk), dC = Mbar * 0.5 (1 - th^2); per lower entry
-// qbar = -(1 - gamma^2) sum_p t_i^T shat sbar_j
-__global__ void k_gnn_loss_node_bwd(int n, int np, int nsys, const int *node_sys, const int *sdim, const int *ptr,
-                                    const int *adj, const float *C, const double *shat, const double *gam,
-                                    const double *T, const double *SB, float *dC, float *qbar) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// qbar = -(1 - gamma^2) sum_p t_i^T shat sbar_j  (a warp per node)
+#define LB_NODES 8
+__global__ void __launch_bounds__(32 * LB_NODES)
+    k_gnn_loss_node_bwd(int n, int np, int nsys, const int *node_sys, const int *sdim, const int *sys_tile,
+                        const double *tile_tr, const int *ptr, const int *adj, const double *th, const double *shat,
+                        const double *gam, const double *T, const double *SB, float *dC, float *qbar) {
+  __shared__ double scale[LB_NODES];
+  int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int i = blockIdx.x * LB_NODES + wid;
+  if (threadIdx.x < LB_NODES && blockIdx.x * LB_NODES + threadIdx.x < n) {
+    int s = node_sys[blockIdx.x * LB_NODES + threadIdx.x];
+    double t = 0.0;
+    for (int b = sys_tile[s]; b < sys_tile[s + 1]; b++) t += tile_tr[b];
+    scale[threadIdx.x] = 2.0 / (t * nsys);
+  }
+  __syncthreads();
   if (i >= n) return;
-  double M[6][6], th[21], Mb[6][6];
-  head_M(C + 21 * (size_t)i, M, th);
-  for (int r = 0; r < 6; r++)
-    for (int c = 0; c < 6; c++) Mb[r][c] = 0.0;
-  for (int a = ptr[i]; a < ptr[i + 1]; a++)
-    if (adj[a] < i) qbar[a] = 0.0f;
-  for (int p = 0; p < np; p++) {
-    const double *ti = T + 6 * ((size_t)i * np + p);
-    double tb[6];
-    for (int k = 0; k < 6; k++) tb[k] = SB[6 * ((size_t)i * np + p) + k];
-    for (int a = ptr[i]; a < ptr[i + 1]; a++) {
+  double cs = scale[wid];
+  int r = min(lane & 7, 5), p0 = lane >> 3;
+  bool row = (lane & 7) < 6;
+  double M[6], tv[6];  // row r of M (c <= r), column r (c > r); tanh of row r
+  for (int c = 0; c < 6; c++) {
+    tv[c] = th[21 * (size_t)i + tri(max(r, c), min(r, c))];
+    M[c] = (c == r ? 1.0 : 0.0) + G_EPS * tv[c];
+  }
+  double inv = 1.0 / ((1.0) + G_EPS * th[21 * (size_t)i + tri(r, r)]);
+  double mb[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int pc = 0; pc < np; pc += 4) {
+    bool on = row && pc + p0 < np;
+    int p = min(pc + p0, np - 1);
+    double ti = on ? T[6 * ((size_t)i * np + p) + r] : 0.0, tb = SB[6 * ((size_t)i * np + p) + r];
+    for (int a = ptr[i], end = ptr[i + 1]; a < end; a++) {
       int j = adj[a];
       if (j >= i) continue;
-      const double *Sh = shat + 36 * (size_t)a;
-      const double *sj = SB + 6 * ((size_t)j * np + p);
-      double gsum = 0.0;
-      for (int r = 0; r < 6; r++) {
-        double t = 0.0;
-        for (int c = 0; c < 6; c++) t += Sh[6 * r + c] * sj[c];
-        tb[r] -= gam[a] * t;
-        gsum += ti[r] * t;
+      const double *Sh = shat + 36 * (size_t)a + 6 * r, *sj = SB + 6 * ((size_t)j * np + p);
+      double t = 0.0, gm = gam[a];
+#pragma unroll
+      for (int c = 0; c < 6; c++) t += Sh[c] * sj[c];
+      tb -= gm * t;
+      t *= ti;
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        float q = -(float)(cs * t * (1.0 - gm * gm));
+        qbar[a] = pc ? qbar[a] + q : q;
       }
-      qbar[a] -= (float)(gsum * (1.0 - gam[a] * gam[a]));
     }
-    fwd_M(M, tb);  // M^-1 tbar
-    for (int r = 0; r < 6; r++)
-      for (int c = 0; c <= r; c++) Mb[r][c] -= ti[r] * tb[c];
+    tb *= cs;
+#pragma unroll
+    for (int c = 0; c < 6; c++) {  // M^-1 tbar
+      if (r == c) tb *= inv;
+      double y = __shfl_sync(0xffffffffu, tb, c, 8);
+      if (r > c) tb -= M[c] * y;
+      mb[c] -= ti * y;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 6; c++) {
+    mb[c] += __shfl_xor_sync(0xffffffffu, mb[c], 8);
+    mb[c] += __shfl_xor_sync(0xffffffffu, mb[c], 16);
   }
   double dd = 2.0 / ((double)sdim[node_sys[i]] * nsys);
-  float *o = dC + 21 * (size_t)i;
-  for (int r = 0; r < 6; r++)
+  if (lane < 6)
     for (int c = 0; c <= r; c++) {
-      double m = Mb[r][c] + (r == c ? dd / M[r][r] : 0.0);
-      double t = th[tri(r, c)];
-      o[tri(r, c)] = (float)(m * G_EPS * (1.0 - t * t));
+      double m = mb[c] + (r == c ? dd * inv : 0.0);
+      dC[21 * (size_t)i + tri(r, c)] = (float)(m * G_EPS * (1.0 - tv[c] * tv[c]));
     }
-}
-
-// edge head backward, one warp per node v: dh_v += sum over v's entries of
-// qbar (ws + wp * h_u); per-node partial gradients of ws, wp, we, bq from the
-// node's lower entries -> EP[v][130]
-__global__ void k_gnn_edge_bwd(int n, const int *ptr, const int *adj, const int *mir, const float *e, const float *h,
-                               const float *w, const float *qbar, float *dh, float *EP) {
-  int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (v >= n) return;
-  const float *hv = h + (size_t)v * GH;
-  float d0 = 0.f, d1 = 0.f, s0 = 0.f, s1 = 0.f, p0 = 0.f, p1 = 0.f, se = 0.f, sb = 0.f;
-  float ws0 = w[G_ws + lane], ws1 = w[G_ws + lane + 32], wp0 = w[G_wp + lane], wp1 = w[G_wp + lane + 32];
-  for (int a = ptr[v]; a < ptr[v + 1]; a++) {
-    int u = adj[a];
-    bool low = u < v;
-    float qb = qbar[low ? a : mir[a]];
-    const float *hu = h + (size_t)u * GH;
-    float hu0 = hu[lane], hu1 = hu[lane + 32];
-    d0 += qb * (ws0 + wp0 * hu0);
-    d1 += qb * (ws1 + wp1 * hu1);
-    if (low) {
-      s0 += qb * (hv[lane] + hu0);
-      s1 += qb * (hv[lane + 32] + hu1);
-      p0 += qb * hv[lane] * hu0;
-      p1 += qb * hv[lane + 32] * hu1;
-      se += qb * e[a];
-      sb += qb;
-    }
-  }
-  dh[(size_t)v * GH + lane] += d0;
-  dh[(size_t)v * GH + lane + 32] += d1;
-  float *o = EP + (size_t)v * G_EDGE_PARAMS;
-  o[lane] = s0;
-  o[lane + 32] = s1;
-  o[GH + lane] = p0;
-  o[GH + lane + 32] = p1;
-  if (lane == 0) {
-    o[2 * GH] = se;
-    o[2 * GH + 1] = sb;
-  }
-}
-
-// out[c] = sum_v in[v][c] in node order
-__global__ void k_gnn_colsum(int n, int ncol, const float *in, float *out) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncol) return;
-  double t = 0.0;
-  for (int v = 0; v < n; v++) t += in[(size_t)v * ncol + c];
-  out[c] = (float)t;
 }
 
 // z[i] ~ N(0, 1) from a counter: splitmix64 (Steele, Lea, Flood 2014) of
@@ -739,22 +1019,20 @@ static rpba_status gnn_forward(KL &kl, const GnnNet &net, const GnnAct &a, cudaS
   int n = a.n;
   if (n == 0) return RPBA_OK;
   int gl = nblk(n, GL_NODES);
-  RPBA_TRY(kl("k_gnn_linear", [&] {
-    k_gnn_linear<false><<<gl, 256, 0, st>>>(n, a.x, GNF, net.wb + G_W0, nullptr, 0, nullptr, net.w + G_b0, GH, 1, 0,
-                                            a.h[0]);
+  RPBA_TRY(kl("k_gnn_layer", [&] {
+    k_gnn_layer<GNF, false, false><<<gl, 256, 0, st>>>(n, nullptr, nullptr, nullptr, a.x, net.wb + G_W0, nullptr,
+                                                       net.w + G_b0, nullptr, a.h[0], nullptr, nullptr, nullptr);
   }));
-  for (int t = 1; t <= GNL; t++) {
-    RPBA_TRY(kl("k_gnn_aggregate", [&] {
-      k_gnn_aggregate<<<nblk((long long)n * 32, 256), 256, 0, st>>>(n, a.ptr, a.adj, a.e, a.h[t - 1], a.m[t - 1], 0);
+  for (int t = 1; t < GNL; t++)
+    RPBA_TRY(kl("k_gnn_layer", [&] {
+      k_gnn_layer<GH, true, false><<<gl, 256, 0, st>>>(n, a.ptr, a.adj, a.e, a.h[t - 1], net.wb + g_A(t),
+                                                       net.wb + g_B(t), net.w + g_c(t), a.m[t - 1], a.h[t], nullptr,
+                                                       nullptr, nullptr);
     }));
-    RPBA_TRY(kl("k_gnn_linear", [&] {
-      k_gnn_linear<false><<<gl, 256, 0, st>>>(n, a.h[t - 1], GH, net.wb + g_A(t), a.m[t - 1], GH, net.wb + g_B(t),
-                                              net.w + g_c(t), GH, 1, 0, a.h[t]);
-    }));
-  }
-  RPBA_TRY(kl("k_gnn_linear", [&] {
-    k_gnn_linear<false><<<gl, 256, 0, st>>>(n, a.h[GNL], GH, net.wb + G_Wo, nullptr, 0, nullptr, net.w + G_bo, GNF, 0,
-                                            0, a.C);
+  RPBA_TRY(kl("k_gnn_layer", [&] {
+    k_gnn_layer<GH, true, true><<<gl, 256, 0, st>>>(n, a.ptr, a.adj, a.e, a.h[GNL - 1], net.wb + g_A(GNL),
+                                                    net.wb + g_B(GNL), net.w + g_c(GNL), a.m[GNL - 1], a.h[GNL],
+                                                    net.wb + G_Wo, net.w + G_bo, a.C);
   }));
   return RPBA_OK;
 }
@@ -1022,10 +1300,11 @@ struct rpba_gnn {
   long long *soff = nullptr;
   float *e = nullptr, *x = nullptr;
   double *L = nullptr, *shat = nullptr, *z = nullptr, *S = nullptr;
-  float *act = nullptr, *C = nullptr, *dC = nullptr, *dh = nullptr, *dz = nullptr, *tmp = nullptr, *part = nullptr,
-        *qbar = nullptr, *EP = nullptr;
-  double *gam = nullptr, *T = nullptr, *V = nullptr, *U = nullptr, *SB = nullptr, *Ts = nullptr, *loss_s = nullptr,
-         *loss = nullptr;
+  float *act = nullptr, *C = nullptr, *dC = nullptr, *dh = nullptr, *tmp = nullptr, *part = nullptr,
+        *qbar = nullptr;
+  double *gam = nullptr, *T = nullptr, *V = nullptr, *SB = nullptr, *th = nullptr, *ld = nullptr, *epart = nullptr,
+         *tile_tr = nullptr, *tile_ld = nullptr, *loss = nullptr;
+  int ntile = 0, *tile0 = nullptr, *sys_tile = nullptr;
   float *D = nullptr, *Li = nullptr, *F = nullptr;
 };
 
@@ -1250,18 +1529,27 @@ rpba_status prepare(rpba_gnn *G) {
   RPBA_TRY(galloc(G, (void **)&G->C, (size_t)n * 21 * sizeof(float)));
   RPBA_TRY(galloc(G, (void **)&G->dC, (size_t)n * 21 * sizeof(float)));
   RPBA_TRY(galloc(G, (void **)&G->dh, (size_t)n * GH * sizeof(float)));
-  RPBA_TRY(galloc(G, (void **)&G->dz, (size_t)n * GH * sizeof(float)));
-  RPBA_TRY(galloc(G, (void **)&G->tmp, (size_t)n * GH * sizeof(float)));
-  RPBA_TRY(galloc(G, (void **)&G->part, (size_t)nblk(n, WG_NODES) * GH * (GH + 1) * sizeof(float)));
+  RPBA_TRY(galloc(G, (void **)&G->tmp, 2 * (size_t)n * GH * sizeof(float)));
+  RPBA_TRY(galloc(G, (void **)&G->part, (size_t)grad_rows(n) * G_PSTRIDE * sizeof(float)));
+  RPBA_TRY(galloc(G, (void **)&G->epart, (size_t)grad_rows(n) * G_EDGE_PARAMS * sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->qbar, nnz * sizeof(float)));
-  RPBA_TRY(galloc(G, (void **)&G->EP, (size_t)n * G_EDGE_PARAMS * sizeof(float)));
   RPBA_TRY(galloc(G, (void **)&G->gam, nnz * sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->T, nv * sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->V, nv * sizeof(double)));
-  RPBA_TRY(galloc(G, (void **)&G->U, nv * sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->SB, nv * sizeof(double)));
-  RPBA_TRY(galloc(G, (void **)&G->Ts, (size_t)G->nsys * sizeof(double)));
-  RPBA_TRY(galloc(G, (void **)&G->loss_s, (size_t)G->nsys * sizeof(double)));
+  RPBA_TRY(galloc(G, (void **)&G->th, 21 * (size_t)n * sizeof(double)));
+  RPBA_TRY(galloc(G, (void **)&G->ld, (size_t)n * sizeof(double)));
+  // tiles of LS_NODES nodes of one system
+  std::vector<int> tile0, sys_tile{0};
+  for (int s = 0; s < G->nsys; s++) {
+    for (int v = G->h_node0[s]; v < G->h_node0[s + 1]; v += LS_NODES) tile0.push_back(v);
+    sys_tile.push_back((int)tile0.size());
+  }
+  G->ntile = (int)tile0.size();
+  RPBA_TRY(put(G, &G->tile0, tile0));
+  RPBA_TRY(put(G, &G->sys_tile, sys_tile));
+  RPBA_TRY(galloc(G, (void **)&G->tile_tr, tile0.size() * sizeof(double)));
+  RPBA_TRY(galloc(G, (void **)&G->tile_ld, tile0.size() * sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->loss, sizeof(double)));
   RPBA_TRY(galloc(G, (void **)&G->D, (size_t)n * 36 * sizeof(float)));
   RPBA_TRY(galloc(G, (void **)&G->Li, (size_t)n * 36 * sizeof(float)));
@@ -1313,68 +1601,42 @@ rpba_status loss_grad(rpba_gnn *G) {
   int n = G->n, np = G->np, ns = G->nsys;
   cudaStream_t st = G->stream;
   GnnAct a = dataset_act(G);
-  int nvp = n * np;
-  RPBA_TRY(kl("k_gnn_loss_t", [&] { k_gnn_loss_t<<<nblk(nvp, 128), 128, 0, st>>>(n, np, G->C, G->z, G->T); }));
+  RPBA_TRY(kl("k_gnn_loss_t", [&] {
+    k_gnn_loss_t<<<nblk(n, LT_NODES), 256, 0, st>>>(n, np, G->C, G->L, G->z, G->th, G->T, G->ld);
+  }));
   RPBA_TRY(kl("k_gnn_loss_v", [&] {
-    k_gnn_loss_v<<<nblk(nvp, 128), 128, 0, st>>>(n, np, G->ptr, G->adj, G->mir, G->L, G->shat, G->gam, G->T, G->V);
+    k_gnn_loss_v<<<nblk(n, 4), 128, 0, st>>>(n, np, G->ptr, G->adj, G->mir, G->L, G->shat, G->gam, G->T, G->V);
   }));
   RPBA_TRY(kl("k_gnn_loss_symv", [&] {
-    k_gnn_loss_symv<<<nblk(6LL * nvp, 128), 128, 0, st>>>(n, np, G->node_sys, G->node0, G->soff, G->sdim, G->S,
-                                                          G->V, G->U);
-  }));
-  RPBA_TRY(kl("k_gnn_loss_sys", [&] {
-    k_gnn_loss_sys<<<ns, 256, 0, st>>>(ns, np, G->node0, G->sdim, G->C, G->L, G->V, G->U, G->Ts, G->loss_s);
-  }));
-  RPBA_TRY(kl("k_gnn_loss_total", [&] { k_gnn_loss_total<<<1, 32, 0, st>>>(ns, G->loss_s, G->loss); }));
-  RPBA_TRY(kl("k_gnn_loss_sbar", [&] {
-    k_gnn_loss_sbar<<<nblk(nvp, 128), 128, 0, st>>>(n, np, ns, G->node_sys, G->L, G->Ts, G->U, G->SB);
+    k_gnn_loss_symv<<<G->ntile, 128, 0, st>>>(G->ntile, np, G->tile0, G->node_sys, G->node0, G->soff, G->sdim, G->S,
+                                              G->L, G->V, G->ld, G->SB, G->tile_tr, G->tile_ld);
   }));
   RPBA_TRY(kl("k_gnn_loss_node_bwd", [&] {
-    k_gnn_loss_node_bwd<<<nblk(n, 64), 64, 0, st>>>(n, np, ns, G->node_sys, G->sdim, G->ptr, G->adj, G->C, G->shat,
-                                                    G->gam, G->T, G->SB, G->dC, G->qbar);
+    k_gnn_loss_node_bwd<<<nblk(n, LB_NODES), 32 * LB_NODES, 0, st>>>(n, np, ns, G->node_sys, G->sdim, G->sys_tile,
+                                                                     G->tile_tr, G->ptr, G->adj, G->th, G->shat,
+                                                                     G->gam, G->T, G->SB, G->dC, G->qbar);
   }));
-  int nw = nblk(n, WG_NODES);
-  auto wgrad = [&](const float *dz, int nout, const float *in, int nin, int offW, int offb) -> rpba_status {
-    RPBA_TRY(kl("k_gnn_wgrad", [&] { k_gnn_wgrad<<<nw, 256, 0, st>>>(n, dz, nout, in, nin, G->part); }));
-    return kl("k_gnn_wgrad_reduce", [&] {
-      k_gnn_wgrad_reduce<<<nblk(nout * (nin + 1), 256), 256, 0, st>>>(nw, nout, nin, G->part, G->g + offW,
-                                                                    G->g + offb);
-    });
-  };
-  int gl = nblk(n, GL_NODES);
-  long long nh = (long long)n * GH;
-  // output heads
-  RPBA_TRY(wgrad(G->dC, GNF, a.h[GNL], GH, G_Wo, G_bo));
-  RPBA_TRY(kl("k_gnn_linear", [&] {
-    k_gnn_linear<true><<<gl, 256, 0, st>>>(n, G->dC, GNF, G->wb + G_Wo, nullptr, 0, nullptr, nullptr, GH, 0, 0, G->dh);
-  }));
-  RPBA_TRY(kl("k_gnn_edge_bwd", [&] {
-    k_gnn_edge_bwd<<<nblk((long long)n * 32, 256), 256, 0, st>>>(n, G->ptr, G->adj, G->mir, G->e, a.h[GNL], G->w,
-                                                                 G->qbar, G->dh, G->EP);
-  }));
-  RPBA_TRY(kl("k_gnn_colsum", [&] {
-    k_gnn_colsum<<<nblk(G_EDGE_PARAMS, 64), 64, 0, st>>>(n, G_EDGE_PARAMS, G->EP, G->g + G_ws);
+  int rows = grad_rows(n);
+  RPBA_TRY(kl("k_gnn_head_bwd", [&] {
+    k_gnn_head_bwd<<<rows, 256, 0, st>>>(n, G->ptr, G->adj, G->mir, G->e, a.h[GNL], G->w, G->wb, G->dC, G->qbar,
+                                         G->dh, G->part, G->epart);
   }));
   for (int t = GNL; t >= 1; t--) {
-    RPBA_TRY(kl("k_gnn_relu_bwd", [&] { k_gnn_relu_bwd<<<nblk(nh, 256), 256, 0, st>>>(nh, G->dh, a.h[t], G->dz); }));
-    RPBA_TRY(wgrad(G->dz, GH, a.h[t - 1], GH, g_A(t), g_c(t)));
-    RPBA_TRY(wgrad(G->dz, GH, a.m[t - 1], GH, g_B(t), g_c(t)));  // the same bias gradient, written twice
-    // dm = B^T dz ; dh_prev = A^T dz + aggregate(dm)
-    RPBA_TRY(kl("k_gnn_linear", [&] {
-      k_gnn_linear<true><<<gl, 256, 0, st>>>(n, G->dz, GH, G->wb + g_B(t), nullptr, 0, nullptr, nullptr, GH, 0, 0,
-                                             G->tmp);
-    }));
-    RPBA_TRY(kl("k_gnn_linear", [&] {
-      k_gnn_linear<true><<<gl, 256, 0, st>>>(n, G->dz, GH, G->wb + g_A(t), nullptr, 0, nullptr, nullptr, GH, 0, 0,
-                                             G->dh);
-    }));
-    RPBA_TRY(kl("k_gnn_aggregate", [&] {
-      k_gnn_aggregate<<<nblk((long long)n * 32, 256), 256, 0, st>>>(n, a.ptr, a.adj, a.e, G->tmp, G->dh, 1);
+    float *in = G->tmp + (size_t)(t & 1) * n * GH, *out = G->tmp + (size_t)(~t & 1) * n * GH;
+    RPBA_TRY(kl("k_gnn_layer_bwd", [&] {
+      auto k = t == GNL ? k_gnn_layer_bwd<GH, false> : k_gnn_layer_bwd<GH, true>;
+      k<<<rows, 256, 0, st>>>(n, a.ptr, a.adj, a.e, a.h[t], G->dh, in, out, a.h[t - 1], a.m[t - 1], G->wb + g_A(t),
+                              G->wb + g_B(t), g_A(t), g_B(t), g_c(t), G->part);
     }));
   }
-  RPBA_TRY(kl("k_gnn_relu_bwd", [&] { k_gnn_relu_bwd<<<nblk(nh, 256), 256, 0, st>>>(nh, G->dh, a.h[0], G->dz); }));
-  RPBA_TRY(wgrad(G->dz, GH, a.x, GNF, G_W0, G_b0));
-  return RPBA_OK;
+  RPBA_TRY(kl("k_gnn_layer_bwd", [&] {
+    k_gnn_layer_bwd<GNF, true><<<rows, 256, 0, st>>>(n, a.ptr, a.adj, a.e, a.h[0], G->dh, G->tmp, nullptr, a.x,
+                                                     nullptr, nullptr, nullptr, G_W0, 0, G_b0, G->part);
+  }));
+  return kl("k_gnn_grad_reduce", [&] {
+    k_gnn_grad_reduce<<<nblk(G_NPARAM, 32) + 1, 256, 0, st>>>(rows, G->part, G->epart, G->g, ns, np, G->sys_tile,
+                                                              G->sdim, G->tile_tr, G->tile_ld, G->loss);
+  });
 }
 
 }  // namespace
