@@ -155,7 +155,7 @@ __device__ __forceinline__ float rcp_ulp(float x) { return __frcp_rn(x); }
 // four schedulers has its own FP64 pipe, 64 cycles per instruction): an FP64
 // tile alone took 93 us by one warp with a square root and a division per
 // column, 57 us without the divisions, 29 us by eight warps (FP32 tile: 24 ->
-// 13 us; launch included). The warp that owns column j + 1 updates it first
+// 19 us; launch included). The warp that owns column j + 1 updates it first
 // and publishes it, scaled by its pivot's reciprocal, while the others work:
 // one barrier per step. Whole factorisations, with the diagonal tiles' CTAs
 // first in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.23 ms,
@@ -672,15 +672,77 @@ __global__ void __launch_bounds__(128) k_chol_tc_persistent(const __grid_constan
 
 // forward L z = r and backward L^T x = z (r in, x out, may alias), one thread
 // block cluster of TS CTAs per sub-block. Tile rows are owned round-robin
-// (tile t by CTA t % TS); each step the owner of tile k solves its 32 entries
-// with the inverted diagonal tile and publishes them in its shared memory,
-// one cluster barrier later every CTA reads them through distributed shared
-// memory and updates the tiles it owns. The barrier is the hardware cluster
-// barrier (no software wait). Two buffers alternate between steps.
+// (tile t by CTA t % TS), z of the owned rows stays in shared memory. Each step
+// the owner of tile k solves its 32 entries with the inverted diagonal tile and
+// stores them into the ring of every CTA (st.async; the bytes complete an
+// mbarrier there); the CTAs update the tiles they own, the owner of tile k + 1
+// that one first, so that it solves and publishes without waiting for the rest.
+//
+// A chain of 2 npad / 32 dependent steps: its length is the time. A cluster
+// barrier, a read of the published entries from the owner's shared memory and z
+// in global memory took 2.4 us per step (32 sub-blocks of 30 tiles, FP32: 145 us
+// with the launch), one store with an mbarrier takes 0.9 us (58 us; FP64, 8
+// sub-blocks of 24 tiles: 158 -> 85 us).
+//
+// The ring needs no release: whoever publishes x_m has read x_{m-2} and all
+// before it, every rank owns one of any TS successive tiles, and x_{k+TR} depends
+// on all of x_{k+TR-TS} .. x_{k+TR-1}. So by then every CTA has published some
+// m >= k + TR - TS and is done with x_k if TR >= TS + 2.
 #define TS 8
+#define TR 16          // slots of the ring
+#define TRSV_PRE 4     // owned tiles of the next step in registers (more are read late)
+#define TRSV_WAIT_NS 500000000ull
+static_assert(TR >= TS + 2, "a slot is free when it is written again");
+
+// thread part of eight: (4 c .. 4 c + 3) . v
+template <typename T>
+__device__ inline T eighth_dot(const T *m, const T *v) {
+  T s = 0;
+#pragma unroll
+  for (int c = 0; c < 4; c++) s += m[c] * v[c];
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 8);
+  return s;
+}
+
+__device__ inline void st_async(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr),
+               "r"(__float_as_uint(v)), "r"(bar)
+               : "memory");
+}
+__device__ inline void st_async(uint32_t addr, double v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr),
+               "l"(__double_as_longlong(v)), "r"(bar)
+               : "memory");
+}
+__device__ inline uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// phase of a barrier that other CTAs of the cluster complete
+__device__ inline bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
+  uint64_t t0 = 0;
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(tc::smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    uint64_t t = tc::global_ns();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > limit_ns) return false;
+  }
+}
+
+static size_t trsv_smem(int tiles, size_t elem) { return (size_t)((tiles + TS - 1) / TS) * CT * elem; }
+
 template <typename T>
 __global__ void __cluster_dims__(TS, 1, 1) __launch_bounds__(256)
-    k_trsv_cluster(const T *S, const T *Linv, CholView cv, const int *voff, T *r, T *x) {
+    k_trsv_cluster(const T *S, const T *Linv, CholView cv, const int *voff, const T *r, T *x) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   int rank = (int)cluster.block_rank();
@@ -690,116 +752,174 @@ __global__ void __cluster_dims__(TS, 1, 1) __launch_bounds__(256)
   int nt = np / CT;
   const T *A = S + cv.off[l];
   const T *LI = Linv + cv.linv_off[l];
-  T *z = r + voff[l];
   T *xo = x + voff[l];
-  __shared__ T buf[2][CT];
-  __shared__ T loc[CT];
+  extern __shared__ __align__(16) unsigned char trsv_dyn[];
+  T *zs = reinterpret_cast<T *>(trsv_dyn);  // owned tile t at (t / TS) CT
+  __shared__ __align__(16) T ring[2][TR][CT];
+  __shared__ __align__(8) uint64_t bar[2][TR];
   int tid = threadIdx.x;
-  int row = tid >> 3, part = tid & 7;  // 32 rows x 8 parts of 4 columns
-  // forward; the L tiles a CTA needs after the barrier of step k are read
-  // into registers before it, so their latency overlaps the barrier
-  const int MAXT = 8;  // owned tiles prefetched per step (more are read late)
+  int row = tid >> 3, part = tid & 7;  // 32 rows (columns going back) x 8 parts of 4
+  static_assert(TS == 8, "part addresses a CTA");
+  if (tid == 0) {
+    for (int i = 0; i < 2 * TR; i++) tc::mbar_init(&bar[0][0] + i, 1);
+    tc::fence_mbar_init();
+    for (int i = 0; i < 2 * TR; i++)
+      if (i % TR < nt) tc::mbar_arrive_expect_tx(&bar[0][0] + i, CT * sizeof(T));
+  }
+  for (int t = rank + TS * (tid >> 5); t < nt; t += TS * 8)
+    zs[(t / TS) * CT + (tid & 31)] = r[voff[l] + t * CT + (tid & 31)];
+  cluster.sync();
+  bool ok = true;
+  auto publish = [&](int dir, int step, T v) {
+    int s = step % TR;
+    st_async(map_rank(tc::smem_u32(&ring[dir][s][row]), part), v, map_rank(tc::smem_u32(&bar[dir][s]), part));
+  };
+  // entries of the step (this thread's four), in place for all CTAs
+  auto receive = [&](int dir, int step, T *xv) {
+    int s = step % TR;
+    if (ok) ok = mbar_wait_cluster(&bar[dir][s], (step / TR) & 1, TRSV_WAIT_NS);
+#pragma unroll
+    for (int c = 0; c < 4; c++) xv[c] = ring[dir][s][part * 4 + c];
+    if (tid == 0 && ok && step + TR < nt) tc::mbar_arrive_expect_tx(&bar[dir][s], CT * sizeof(T));
+  };
+  T li[4], pre[TRSV_PRE][4], xv[4];
+  // forward: tiles t0 + m TS of column k below the diagonal
+  auto first_below = [&](int k) { return k + 1 + ((rank - (k + 1)) % TS + TS) % TS; };
+  auto load_tile = [&](int t, int k, T *d) {
+    const T *Lt = A + (size_t)(t * CT + row) * np + k * CT + part * 4;
+#pragma unroll
+    for (int c = 0; c < 4; c++) d[c] = Lt[c];
+  };
+  auto load_li = [&](int t) {
+    if (t < nt)
+#pragma unroll
+      for (int c = 0; c < 4; c++) li[c] = LI[(size_t)t * CT * CT + row * CT + part * 4 + c];
+  };
+  load_li(rank);
+  {
+    int t0 = first_below(0);
+#pragma unroll
+    for (int m = 0; m < TRSV_PRE; m++)
+      if (t0 + m * TS < nt) load_tile(t0 + m * TS, 0, pre[m]);
+  }
+  if (rank == 0) {
+    publish(0, 0, eighth_dot(li, zs + part * 4));
+    load_li(TS);
+  }
   for (int k = 0; k < nt; k++) {
-    int owner = k % TS;
-    int t0 = k + 1 + ((rank - (k + 1)) % TS + TS) % TS;
-    T pre[MAXT][4];
+    T nxt[TRSV_PRE][4];
+    int t0 = first_below(k), t1 = first_below(k + 1);
 #pragma unroll
-    for (int m = 0; m < MAXT; m++) {
+    for (int m = 0; m < TRSV_PRE; m++)
+      if (t1 + m * TS < nt) load_tile(t1 + m * TS, k + 1, nxt[m]);
+    receive(0, k, xv);
+    // the solved entries replace z_k: every thread of this CTA has read it before
+    // its row's entry was published
+    if (rank == k % TS && tid < CT) zs[(k / TS) * CT + tid] = ring[0][k % TR][tid];
+#pragma unroll
+    for (int m = 0; m < TRSV_PRE; m++) {
       int t = t0 + m * TS;
       if (t < nt) {
-        const T *Lt = A + (size_t)(t * CT + row) * np + k * CT + part * 4;
-#pragma unroll
-        for (int c = 0; c < 4; c++) pre[m][c] = Lt[c];
+        T s = eighth_dot(pre[m], xv);
+        if (part == 0) zs[(t / TS) * CT + row] -= s;
+        if (m == 0 && t == k + 1) {
+          __syncthreads();
+          publish(0, t, eighth_dot(li, zs + (t / TS) * CT + part * 4));
+          load_li(t + TS);
+        }
       }
     }
-    if (rank == owner) {
-      const T *Li = LI + (size_t)k * CT * CT;
-      T s = 0;
+    for (int tg = t0 + TRSV_PRE * TS; tg < nt; tg += TRSV_PRE * TS) {
+      T d[TRSV_PRE][4];
 #pragma unroll
-      for (int c = 0; c < 4; c++) s += Li[row * CT + part * 4 + c] * z[k * CT + part * 4 + c];
-      for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-      if (part == 0) {
-        buf[k & 1][row] = s;
-        z[k * CT + row] = s;
-      }
+      for (int m = 0; m < TRSV_PRE; m++)
+        if (tg + m * TS < nt) load_tile(tg + m * TS, k, d[m]);
+#pragma unroll
+      for (int m = 0; m < TRSV_PRE; m++)
+        if (tg + m * TS < nt) {
+          T s = eighth_dot(d[m], xv);
+          if (part == 0) zs[((tg + m * TS) / TS) * CT + row] -= s;
+        }
     }
-    cluster.sync();
-    const T *src = cluster.map_shared_rank(&buf[k & 1][0], owner);
-    if (tid < CT) loc[tid] = src[tid];
-    __syncthreads();
 #pragma unroll
-    for (int m = 0; m < MAXT; m++) {
-      int t = t0 + m * TS;
-      if (t < nt) {
-        T s = 0;
+    for (int m = 0; m < TRSV_PRE; m++)
 #pragma unroll
-        for (int c = 0; c < 4; c++) s += pre[m][c] * loc[part * 4 + c];
-        for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-        if (part == 0) z[t * CT + row] -= s;
-      }
-    }
-    for (int t = t0 + MAXT * TS; t < nt; t += TS) {
-      const T *Lt = A + (size_t)(t * CT + row) * np + k * CT + part * 4;
-      T s = 0;
-#pragma unroll
-      for (int c = 0; c < 4; c++) s += Lt[c] * loc[part * 4 + c];
-      for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-      if (part == 0) z[t * CT + row] -= s;
-    }
-    __syncthreads();
+      for (int c = 0; c < 4; c++) pre[m][c] = nxt[m][c];
   }
-  // backward
+  __syncthreads();
+  // backward: z_t -= L_kt^T x_k, tiles t0 - m TS of row k left of the diagonal
+  auto last_left = [&](int k) { return k - 1 - ((k - 1 - rank) % TS + TS) % TS; };
+  auto load_tile_t = [&](int t, int k, T *d) {
+    const T *Lt = A + (size_t)(k * CT + part * 4) * np + t * CT + row;
+#pragma unroll
+    for (int c = 0; c < 4; c++) d[c] = Lt[(size_t)c * np];
+  };
+  auto load_lit = [&](int t) {
+    if (t >= 0)
+#pragma unroll
+      for (int c = 0; c < 4; c++) li[c] = LI[(size_t)t * CT * CT + (part * 4 + c) * CT + row];
+  };
+  auto solve_back = [&](int t) {
+    T s = eighth_dot(li, zs + (t / TS) * CT + part * 4);
+    publish(1, nt - 1 - t, s);
+    if (part == 0) xo[t * CT + row] = s;
+    load_lit(t - TS);
+  };
+  load_lit(last_left(nt));
+  {
+    int t0 = last_left(nt - 1);
+#pragma unroll
+    for (int m = 0; m < TRSV_PRE; m++)
+      if (t0 - m * TS >= 0) load_tile_t(t0 - m * TS, nt - 1, pre[m]);
+  }
+  if (nt && rank == (nt - 1) % TS) solve_back(nt - 1);
   for (int k = nt - 1; k >= 0; k--) {
-    int owner = k % TS;
-    int col = tid >> 3;
-    T pre[MAXT][4];
+    T nxt[TRSV_PRE][4];
+    int t0 = last_left(k), t1 = last_left(k - 1);
 #pragma unroll
-    for (int m = 0; m < MAXT; m++) {
-      int t = rank + m * TS;
-      if (t < k) {
-        const T *Lt = A + (size_t)(k * CT + part * 4) * np + t * CT + col;
+    for (int m = 0; m < TRSV_PRE; m++)
+      if (t1 - m * TS >= 0) load_tile_t(t1 - m * TS, k - 1, nxt[m]);
+    receive(1, nt - 1 - k, xv);
 #pragma unroll
-        for (int rr = 0; rr < 4; rr++) pre[m][rr] = Lt[(size_t)rr * np];
+    for (int m = 0; m < TRSV_PRE; m++) {
+      int t = t0 - m * TS;
+      if (t >= 0) {
+        T s = eighth_dot(pre[m], xv);
+        if (part == 0) zs[(t / TS) * CT + row] -= s;
+        if (m == 0 && t == k - 1) {
+          __syncthreads();
+          solve_back(t);
+        }
       }
     }
-    if (rank == owner) {
-      const T *Li = LI + (size_t)k * CT * CT;
-      T s = 0;
+    for (int tg = t0 - TRSV_PRE * TS; tg >= 0; tg -= TRSV_PRE * TS) {
+      T d[TRSV_PRE][4];
 #pragma unroll
-      for (int c = 0; c < 4; c++) s += Li[(part * 4 + c) * CT + row] * z[k * CT + part * 4 + c];
-      for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-      if (part == 0) {
-        buf[k & 1][row] = s;
-        xo[k * CT + row] = s;
-      }
+      for (int m = 0; m < TRSV_PRE; m++)
+        if (tg - m * TS >= 0) load_tile_t(tg - m * TS, k, d[m]);
+#pragma unroll
+      for (int m = 0; m < TRSV_PRE; m++)
+        if (tg - m * TS >= 0) {
+          T s = eighth_dot(d[m], xv);
+          if (part == 0) zs[((tg - m * TS) / TS) * CT + row] -= s;
+        }
     }
-    cluster.sync();
-    const T *src = cluster.map_shared_rank(&buf[k & 1][0], owner);
-    if (tid < CT) loc[tid] = src[tid];
-    __syncthreads();
-    // z_j -= L_kj^T x_k for owned tiles j < k: column c of the tile, 8 parts of 4 rows
 #pragma unroll
-    for (int m = 0; m < MAXT; m++) {
-      int t = rank + m * TS;
-      if (t < k) {
-        T s = 0;
+    for (int m = 0; m < TRSV_PRE; m++)
 #pragma unroll
-        for (int rr = 0; rr < 4; rr++) s += pre[m][rr] * loc[part * 4 + rr];
-        for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-        if (part == 0) z[t * CT + col] -= s;
-      }
-    }
-    for (int t = rank + MAXT * TS; t < k; t += TS) {
-      const T *Lt = A + (size_t)(k * CT + part * 4) * np + t * CT + col;
-      T s = 0;
-#pragma unroll
-      for (int rr = 0; rr < 4; rr++) s += Lt[(size_t)rr * np] * loc[part * 4 + rr];
-      for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 8);
-      if (part == 0) z[t * CT + col] -= s;
-    }
-    __syncthreads();
+      for (int c = 0; c < 4; c++) pre[m][c] = nxt[m][c];
   }
-  cluster.sync();  // keep every CTA's shared memory alive until all reads are done
+  if (!ok) cv.fail[l] = 1;
+  cluster.sync();  // stores into this CTA's ring are in before it leaves
+}
+
+template <typename T>
+static rpba_status trsv(Ctx *ctx, const char *name, const T *S, const T *Linv, const CholView &cv, T *r) {
+  size_t smem = trsv_smem(ctx->max_tiles, sizeof(T));
+  if (smem > 32 * 1024)  // beyond this the ring and z need more than the default 48 KB
+    RPBA_CUDA(cudaFuncSetAttribute(k_trsv_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RPBA_KERNEL(ctx, name, k_trsv_cluster<T><<<dim3(TS, ctx->L), 256, smem, ctx->stream>>>(S, Linv, cv, ctx->ycam_off, r, r));
+  return RPBA_OK;
 }
 
 template <typename T>
@@ -1066,8 +1186,7 @@ rpba_status launch_solve_rcs(Ctx *ctx, const int *run_dev, int *fail_dev) {
     CholView cv{ctx->S_off, ctx->npad, ctx->linv_off, run_dev, fail_dev, ctx->sched, ctx->L};
     RPBA_TRY(factor<double>(ctx, ctx->S, ctx->Linv64, cv, T_max));
     RPBA_CUDA(cudaMemcpyAsync(ctx->dC, ctx->y, ctx->ytot * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
-    RPBA_KERNEL(ctx, "k_trsv_f64", k_trsv_cluster<double><<<dim3(TS, ctx->L), 256, 0, ctx->stream>>>(
-                                     ctx->S, ctx->Linv64, cv, ctx->ycam_off, ctx->dC, ctx->dC));
+    RPBA_TRY(trsv<double>(ctx, "k_trsv_f64", ctx->S, ctx->Linv64, cv, ctx->dC));
     return RPBA_OK;
   }
   // mixed: FP32 factor of the scaled system, FP64 iterative refinement
@@ -1096,8 +1215,7 @@ rpba_status launch_solve_rcs(Ctx *ctx, const int *run_dev, int *fail_dev) {
     RPBA_KERNEL(ctx, "k_mixed_residual",
                 k_mixed_residual<<<g, 256, 0, ctx->stream>>>(run_dev, fail_dev, ctx->ycam_off, ctx->npad, ctx->L,
                                                              ctx->ir_rs, ctx->ir_d, ctx->ir_t, ctx->ir_r32, it == 0));
-    RPBA_KERNEL(ctx, "k_trsv_f32", k_trsv_cluster<float><<<dim3(TS, ctx->L), 256, 0, ctx->stream>>>(
-                                     ctx->S32, ctx->Linv32, cv, ctx->ycam_off, ctx->ir_r32, ctx->ir_r32));
+    RPBA_TRY(trsv<float>(ctx, "k_trsv_f32", ctx->S32, ctx->Linv32, cv, ctx->ir_r32));
     RPBA_KERNEL(ctx, "k_mixed_update",
                 k_mixed_update<<<g, 256, 0, ctx->stream>>>(run_dev, fail_dev, ctx->ycam_off, ctx->npad, ctx->L,
                                                            ctx->ir_r32, ctx->ir_x, ctx->ir_d, ctx->dC,
