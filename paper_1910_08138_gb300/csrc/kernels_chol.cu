@@ -68,44 +68,27 @@ __device__ inline int sched_find(const int *base, int L, int idx, int *local) {
   return lo;
 }
 
-// 1 / sqrt(x) to about an ulp
-__device__ __forceinline__ double rsqrt_ulp(double x) { return rsqrt(x); }
-__device__ __forceinline__ float rsqrt_ulp(float x) {
-  float r = rsqrtf(x);
-  float e = fmaf(-x * r, r, 1.f);  // one Newton step
-  return fmaf(0.5f * r, e, r);
-}
-
 // ---------------------------------------------------------------------------
 // one warp: factor the 32 x 32 tile held as rows in registers (lane = row),
 // then invert the factor into smem Xs (row-major, CLD stride). Returns false on
 // a non-positive pivot (uniform across the warp).
-// The factorisation waits for this warp at every step, so it is a short chain:
-// one reciprocal square root per column (the next column's pivot is updated
-// first, so its root overlaps the rest of the update), no divisions, and the
-// inverse column by column with independent updates. The entries above the
-// diagonal are updated too (they are never read): a predicate per entry costs
-// as much as the update.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ bool warp_potrf_inv(T (&x)[CT], T *Ls, T *Xs) {
   int lane = threadIdx.x & 31;
   bool ok = true;
-  T rd = T(0);  // lane j: 1 / L_jj
-  T piv = __shfl_sync(0xffffffffu, x[0], 0);
 #pragma unroll
   for (int j = 0; j < CT; j++) {
+    T piv = __shfl_sync(0xffffffffu, x[j], j);
     if (!(piv > T(0))) ok = false;
-    T r = rsqrt_ulp(piv);
-    if (lane == j) rd = r;
-    T lj = x[j] * r;  // lane j: sqrt(piv)
-    x[j] = lj;
-    if (j + 1 < CT) {
-      x[j + 1] -= lj * __shfl_sync(0xffffffffu, lj, j + 1);
-      piv = __shfl_sync(0xffffffffu, x[j + 1], j + 1);
-    }
+    T d = sqrt(piv);
+    T lj = (lane == j) ? d : x[j] / d;  // L[lane][j] for lane >= j
+    if (lane >= j) x[j] = lj;
 #pragma unroll
-    for (int c = j + 2; c < CT; c++) x[c] -= lj * __shfl_sync(0xffffffffu, lj, c);
+    for (int c = j + 1; c < CT; c++) {
+      T lcj = __shfl_sync(0xffffffffu, lj, c);  // L[c][j]
+      if (lane >= c) x[c] -= lj * lcj;
+    }
   }
   ok = __all_sync(0xffffffffu, ok);
   if (!ok) return false;
@@ -114,16 +97,16 @@ __device__ bool warp_potrf_inv(T (&x)[CT], T *Ls, T *Xs) {
   for (int c = 0; c < CT; c++) Ls[lane * CLD + c] = (c <= lane) ? x[c] : T(0);
   __syncwarp();
   // inverse, column `lane`: forward substitution L xcol = e_lane
+  T xc[CT];
 #pragma unroll
-  for (int r = 0; r < CT; r++) x[r] = (r == lane) ? T(1) : T(0);
+  for (int r = 0; r < CT; r++) {
+    T s = (r == lane) ? T(1) : T(0);
 #pragma unroll
-  for (int m = 0; m < CT; m++) {
-    x[m] *= __shfl_sync(0xffffffffu, rd, m);
-#pragma unroll
-    for (int r = m + 1; r < CT; r++) x[r] -= Ls[r * CLD + m] * x[m];
+    for (int m = 0; m < r; m++) s -= Ls[r * CLD + m] * xc[m];
+    xc[r] = (r >= lane) ? s / Ls[r * CLD + r] : T(0);
   }
 #pragma unroll
-  for (int r = 0; r < CT; r++) Xs[r * CLD + lane] = x[r];
+  for (int r = 0; r < CT; r++) Xs[r * CLD + lane] = xc[r];
   __syncwarp();
   return true;
 }
@@ -140,40 +123,48 @@ __device__ __forceinline__ double rcp_ulp(double x) {
   r = fma(fma(t, t, t), r, r);
   return r * __hiloint2double((2046 - e) << 20, 0);  // 2^(1023 - e)
 }
-__device__ __forceinline__ float rcp_ulp(float x) { return __frcp_rn(x); }
 
 // ---------------------------------------------------------------------------
 // The inverse Cholesky factor of a 32 x 32 SPD tile (smem C, CLD stride, both
 // triangles of the part used: the lower one), by the whole CTA (256 threads),
 // into out (row-major, CT stride). False (uniform) on a non-positive pivot.
-// Elimination of [C | I] without square roots, C = L D L^T with unit L, gives
-// L^-1 beside it; the rows are scaled by D^-1/2 at the end. Thread (row =
-// lane, warp w) holds columns w, w + 8, w + 16, w + 24 of both halves: at step
-// j a column c > j is updated in C, a column c <= j in I, so every step does
-// the same 32 x 32 updates. The factorisation's next step waits for this
-// tile, and one warp alone gets a quarter of the SM's FP64 rate (each of the
-// four schedulers has its own FP64 pipe, 64 cycles per instruction): an FP64
-// tile alone took 93 us by one warp with a square root and a division per
-// column, 57 us without the divisions, 29 us by eight warps (FP32 tile: 24 ->
-// 19 us; launch included). The warp that owns column j + 1 updates it first
-// and publishes it, scaled by its pivot's reciprocal, while the others work:
-// one barrier per step. Whole factorisations, with the diagonal tiles' CTAs
-// first in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.23 ms,
-// eight of 750 3.2 -> 1.7 ms (FP64).
+// Elimination of [C | I] gives L^-1 beside the factor. The factorisation's next
+// step waits for this tile.
+//
+// FP64: without square roots, C = L D L^T with unit L and one reciprocal per
+// step, the rows scaled by D^-1/2 at the end. Thread (row = lane, warp w) holds
+// columns w, w + 8, w + 16, w + 24 of both halves: at step j a column c > j is
+// updated in C, a column c <= j in I, so every step does the same 32 x 32
+// updates. The warp that owns column j + 1 updates it first and publishes it
+// while the others work: one barrier per step. One warp alone gets a quarter of
+// the SM's FP64 rate (each of the four schedulers has its own FP64 pipe, 64
+// cycles per instruction): a tile took 93 us by one warp with a square root and
+// a division per column, 57 us without the divisions, 29 us by eight warps
+// (launch included). Whole factorisations, with the diagonal tiles' CTAs first
+// in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.23 ms, eight of
+// 750 3.2 -> 1.7 ms.
+//
+// FP32: square root and division per column, each entry's operations in the
+// order of warp_potrf_inv, so both give the same bits: the refinement of a badly
+// conditioned block does not remove the last digits of another rounding (5e-8 of
+// a coordinate was seen). Bound by the chain of 32 roots and quotients, so a warp
+// takes 8 columns in registers without a barrier, four warps the four column
+// blocks, the other four the inverse: one barrier per 8 columns, a reciprocal per
+// column. Steps of 32 sub-blocks of up to 38 cameras, which this chain decides: 30 us
+// with a column per barrier, 19 us like this.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ bool cta_inverse_factor(const T *C, T *out) {
-  __shared__ T lcol[2][CT], dv[CT];
+__device__ bool cta_inverse_factor(const double *C, double *out) {
+  __shared__ double lcol[2][CT], dv[CT];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  T a[4], e[4];
+  double a[4], e[4];
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     int c = w + 8 * i;
     a[i] = lane >= c ? C[lane * CLD + c] : C[c * CLD + lane];
-    e[i] = lane == c ? T(1) : T(0);
+    e[i] = lane == c ? 1.0 : 0.0;
   }
-  auto publish = [&](int j, T aj) {  // column j's multipliers, by its owner warp
-    T d = __shfl_sync(0xffffffffu, aj, j);
+  auto publish = [&](int j, double aj) {  // column j's multipliers, by its owner warp
+    double d = __shfl_sync(0xffffffffu, aj, j);
     lcol[j & 1][lane] = aj * rcp_ulp(d);
     if (lane == 0) dv[j] = d;
   };
@@ -184,7 +175,7 @@ __device__ bool cta_inverse_factor(const T *C, T *out) {
     for (int jw = 0; jw < 8; jw++) {
       const int j = 8 * jb + jw;
       __syncthreads();
-      const T l = lane > j ? lcol[j & 1][lane] : T(0);
+      const double l = lane > j ? lcol[j & 1][lane] : 0.0;
       // column j + 1 first, by its owner
       const bool own = j + 1 < CT && w == ((j + 1) & 7);
       if (own) {
@@ -201,19 +192,91 @@ __device__ bool cta_inverse_factor(const T *C, T *out) {
         const int c = w + 8 * i;
         if (c == j + 1) continue;  // done above (the whole warp)
         const bool left = c > j;
-        T v = left ? a[i] : e[i];
+        double v = left ? a[i] : e[i];
         v -= l * __shfl_sync(0xffffffffu, v, j);
         if (left) a[i] = v; else e[i] = v;
       }
     }
   }
   __syncthreads();
-  const T d = dv[lane];
-  const bool ok = __all_sync(0xffffffffu, d > T(0));
+  const double d = dv[lane];
+  const bool ok = __all_sync(0xffffffffu, d > 0.0);
   if (!ok) return false;
-  const T rs = rsqrt_ulp(d);
+  const double rs = rsqrt(d);
 #pragma unroll
   for (int i = 0; i < 4; i++) out[lane * CT + w + 8 * i] = e[i] * rs;
+  return true;
+}
+
+// a / d for the divisor's correctly rounded reciprocal r: two corrections by the
+// exact remainder give the correctly rounded quotient (P. Markstein, IA-64 and
+// Elementary Functions, 2000, ch. 8); the same bits as a / d in 1e9 random pairs
+// without subnormal remainders
+__device__ __forceinline__ float div_by(float a, float d, float r) {
+  float q = a * r;
+  q = fmaf(fmaf(-q, d, a), r, q);
+  return fmaf(fmaf(-q, d, a), r, q);
+}
+
+__device__ bool cta_inverse_factor(const float *C, float *out) {
+  __shared__ float Ls[CT][CT];  // column j of L
+  __shared__ float dg[CT], rdg[CT];
+  __shared__ int bad;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float x[8];  // warps 0 .. 3: columns 8 w + i of C; 4 .. 7: 8 (w - 4) + i of I (row = lane)
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    int c = 8 * (w & 3) + i;
+    x[i] = w < 4 ? (lane >= c ? C[lane * CLD + c] : 0.f) : (lane == c ? 1.f : 0.f);
+  }
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+#pragma unroll 1
+  for (int b = 0; b < 4; b++) {
+    if (w == b) {  // factor the columns 8 b .. 8 b + 7
+      bool ok = true;
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int j = 8 * b + i;
+        float piv = __shfl_sync(0xffffffffu, x[i], j);
+        if (!(piv > 0.f)) ok = false;
+        float d = sqrtf(piv), r = __frcp_rn(d);
+        float l = lane == j ? d : div_by(x[i], d, r);
+        Ls[j][lane] = l;
+        if (lane == i) dg[j] = d, rdg[j] = r;
+#pragma unroll
+        for (int c = i + 1; c < 8; c++) x[c] -= l * __shfl_sync(0xffffffffu, l, 8 * b + c);
+      }
+      if (!ok && lane == 0) bad = 1;
+    }
+    __syncthreads();
+    if (w < 4) {
+      if (w > b)
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const float *L = Ls[8 * b + i];
+          float l = L[lane];
+#pragma unroll
+          for (int c = 0; c < 8; c++) x[c] -= l * L[8 * w + c];
+        }
+    } else if (w - 4 <= b) {  // rows 8 b .. 8 b + 7 of the inverse, and their part of the rows below
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int j = 8 * b + i;
+        const float l = lane > j ? Ls[j][lane] : 0.f, d = dg[j], r = rdg[j];
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+          float y = div_by(__shfl_sync(0xffffffffu, x[c], j), d, r);
+          if (lane == j) x[c] = y;
+          x[c] -= l * y;
+        }
+      }
+    }
+  }
+  if (bad) return false;
+  if (w >= 4)
+#pragma unroll
+    for (int i = 0; i < 8; i++) out[lane * CT + 8 * (w - 4) + i] = x[i];
   return true;
 }
 
@@ -226,7 +289,7 @@ __global__ void __launch_bounds__(256) k_chol_first(T *S, T *Linv, CholView cv) 
   __shared__ T C[CT * CLD];
   for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) C[(e / CT) * CLD + e % CT] = A[(size_t)(e / CT) * np + e % CT];
   __syncthreads();
-  if (!cta_inverse_factor<T>(C, Linv + cv.linv_off[l]) && threadIdx.x == 0) cv.fail[l] = 1;
+  if (!cta_inverse_factor(C, Linv + cv.linv_off[l]) && threadIdx.x == 0) cv.fail[l] = 1;
 }
 
 // 32 x 32 x 32 product on 256 threads, 2 x 2 outputs per thread:
@@ -325,7 +388,7 @@ __global__ void __launch_bounds__(256, 3) k_chol_update(T *S, T *Linv, CholView 
       P[rr * CLD + cc] = A[(size_t)(ti * CT + rr) * np + tj * CT + cc] - acc[r][c];
     }
   __syncthreads();
-  if (!cta_inverse_factor<T>(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT) && threadIdx.x == 0) cv.fail[l] = 1;
+  if (!cta_inverse_factor(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT) && threadIdx.x == 0) cv.fail[l] = 1;
 }
 
 // ---------------------------------------------------------------------------
