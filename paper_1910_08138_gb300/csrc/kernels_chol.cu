@@ -44,7 +44,7 @@ struct CholView {
   const int *linv_off;   // per sub-block offset of its inverted diagonal tiles (elements)
   const int *run;
   int *fail;
-  const int *sched;      // per step k: L+1 prefix sums of panel tiles, then L+1 of update tiles
+  const int *sched;      // per step k: L+1 prefix sums of panel tiles, of update tiles and of 2 x 2 blocks of them
   int L;
 };
 
@@ -323,7 +323,7 @@ __device__ inline void load_tile(T *dst, const T *A, int np, int ti, int tj) {
 template <typename T>
 __global__ void __launch_bounds__(256) k_chol_panel(T *S, const T *Linv, CholView cv, int k) {
   int loc;
-  int l = sched_find(cv.sched + (size_t)k * 2 * (cv.L + 1), cv.L, blockIdx.x, &loc);
+  int l = sched_find(cv.sched + (size_t)k * 3 * (cv.L + 1), cv.L, blockIdx.x, &loc);
   if (!cv.run[l] || cv.fail[l]) return;
   int np = cv.npad[l];
   int nt = np / CT;
@@ -344,51 +344,85 @@ __global__ void __launch_bounds__(256) k_chol_panel(T *S, const T *Linv, CholVie
     for (int c = 0; c < 2; c++) A[(size_t)(ti * CT + ty + 16 * r) * np + k * CT + tx + 16 * c] = acc[r][c];
 }
 
-// The first L CTAs take the sub-blocks' next diagonal tiles, whose factor the
-// next step waits for, so that it overlaps the other tiles' updates.
+// Trailing update: a CTA takes B x B tiles (rows and columns k + 1 + B a .., on or
+// below the diagonal). The first L CTAs take the sub-blocks' next diagonal tiles,
+// whose factor the next step waits for, so that it overlaps the other tiles'
+// updates.
+//
+// B = 2 in FP32: a tile per CTA is a short chain (load, product, store) of 4 outputs
+// per thread, and 32 sub-blocks of 29 tiles are 13,000 CTAs in the first step; 16
+// outputs per thread halve the loads per product and quarter the CTAs (30 steps:
+// 1.29 -> 0.88 ms). Where the diagonal tile's chain decides a step (small
+// sub-blocks) the two are alike (20 steps: 0.38 and 0.35 ms).
+// B = 1 in FP64: bound by its multiply-adds (8 sub-blocks of 24 tiles: 1.2 ms per
+// factorisation of 0.95 ms of them), so larger blocks only lengthen the last wave.
 template <typename T>
-__global__ void __launch_bounds__(256, 3) k_chol_update(T *S, T *Linv, CholView cv, int k) {
-  int loc = 0, l = blockIdx.x;
-  if (l >= cv.L) {
-    l = sched_find(cv.sched + (size_t)k * 2 * (cv.L + 1) + (cv.L + 1), cv.L, blockIdx.x - cv.L, &loc);
-    if (loc == 0) return;  // a diagonal tile
-  }
-  if (!cv.run[l] || cv.fail[l]) return;
-  int np = cv.npad[l];
-  int nt = np / CT;
-  int rem = nt - k - 1;
-  if (rem <= 0) return;
-  int a, b;
-  tri_index(loc, a, b);
-  if (a >= rem) return;
-  int ti = k + 1 + a, tj = k + 1 + b;
-  T *A = S + cv.off[l];
-  __shared__ T P[CT * CLD], Q[CT * CLD];
-  load_tile<T>(P, A, np, ti, k);
-  load_tile<T>(Q, A, np, tj, k);
-  __syncthreads();
-  T acc[2][2];
-  tile_nt<T>(P, Q, acc);
+constexpr int update_block = sizeof(T) == 4 ? 2 : 1;
+template <typename T>
+__global__ void __launch_bounds__(256, 4) k_chol_update(T *S, T *Linv, CholView cv, int k) {
+  constexpr int B = update_block<T>, RB = B * CT, NR = 2 * B;  // NR x NR outputs per thread, 16 apart
   int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  bool diag_next = (ti == k + 1) && (tj == k + 1);
-  if (!diag_next) {
+  __shared__ T P[RB * CLD], Q[RB * CLD];
+  if ((int)blockIdx.x < cv.L) {
+    int l = blockIdx.x;
+    if (!cv.run[l] || cv.fail[l]) return;
+    int np = cv.npad[l];
+    if (k + 1 >= np / CT) return;
+    T *A = S + cv.off[l];
+    load_tile<T>(P, A, np, k + 1, k);
+    __syncthreads();
+    T acc[2][2];
+    tile_nt<T>(P, P, acc);
+    __syncthreads();  // every thread is done with P
 #pragma unroll
     for (int r = 0; r < 2; r++)
 #pragma unroll
-      for (int c = 0; c < 2; c++) A[(size_t)(ti * CT + ty + 16 * r) * np + tj * CT + tx + 16 * c] -= acc[r][c];
+      for (int c = 0; c < 2; c++) {
+        int rr = ty + 16 * r, cc = tx + 16 * c;
+        P[rr * CLD + cc] = A[(size_t)((k + 1) * CT + rr) * np + (k + 1) * CT + cc] - acc[r][c];
+      }
+    __syncthreads();
+    if (!cta_inverse_factor(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT) && threadIdx.x == 0)
+      cv.fail[l] = 1;
     return;
   }
-  // tile (k+1, k+1) is complete: update it and form its inverse factor here
-  __syncthreads();  // every thread is done with P
-#pragma unroll
-  for (int r = 0; r < 2; r++)
-#pragma unroll
-    for (int c = 0; c < 2; c++) {
-      int rr = ty + 16 * r, cc = tx + 16 * c;
-      P[rr * CLD + cc] = A[(size_t)(ti * CT + rr) * np + tj * CT + cc] - acc[r][c];
-    }
+  int loc, l = sched_find(cv.sched + ((size_t)k * 3 + B) * (cv.L + 1), cv.L, blockIdx.x - cv.L, &loc);
+  if (B == 1 && loc == 0) return;  // a diagonal tile
+  if (!cv.run[l] || cv.fail[l]) return;
+  int np = cv.npad[l];
+  int a, b;
+  tri_index(loc, a, b);
+  int r0 = (k + 1 + B * a) * CT, c0 = (k + 1 + B * b) * CT;  // first row and column
+  if (r0 >= np) return;
+  T *A = S + cv.off[l];
+  for (int e = threadIdx.x; e < RB * CT; e += 256) {
+    int r = e / CT, c = e - r * CT;
+    P[r * CLD + c] = r0 + r < np ? A[(size_t)(r0 + r) * np + k * CT + c] : T(0);
+    Q[r * CLD + c] = c0 + r < np ? A[(size_t)(c0 + r) * np + k * CT + c] : T(0);
+  }
   __syncthreads();
-  if (!cta_inverse_factor(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT) && threadIdx.x == 0) cv.fail[l] = 1;
+  T acc[NR][NR] = {};
+#pragma unroll 4
+  for (int m = 0; m < CT; m++) {
+    T p[NR], q[NR];
+#pragma unroll
+    for (int i = 0; i < NR; i++) {
+      p[i] = P[(ty + 16 * i) * CLD + m];
+      q[i] = Q[(tx + 16 * i) * CLD + m];
+    }
+#pragma unroll
+    for (int r = 0; r < NR; r++)
+#pragma unroll
+      for (int c = 0; c < NR; c++) acc[r][c] = fma(p[r], q[c], acc[r][c]);
+  }
+#pragma unroll
+  for (int r = 0; r < NR; r++)
+#pragma unroll
+    for (int c = 0; c < NR; c++) {
+      int ti = B * a + r / 2, tj = B * b + c / 2;  // tiles from k + 1; (0, 0) is the diagonal CTA's
+      if (tj > ti || (ti | tj) == 0 || r0 + 32 * (r / 2) >= np) continue;
+      A[(size_t)(r0 + ty + 16 * r) * np + c0 + tx + 16 * c] -= acc[r][c];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -992,8 +1026,8 @@ static rpba_status factor(Ctx *ctx, T *S, T *Linv, CholView cv, int T_max) {
   const char *n_upd = sizeof(T) == 8 ? "k_chol_update_f64" : "k_chol_update_f32";
   RPBA_KERNEL(ctx, n_first, k_chol_first<T><<<ctx->L, 256, 0, ctx->stream>>>(S, Linv, cv));
   for (int k = 0; k + 1 < T_max; k++) {
-    int np_k = ctx->h_sched[(size_t)k * 2 * (ctx->L + 1) + ctx->L];
-    int nu_k = ctx->h_sched[(size_t)k * 2 * (ctx->L + 1) + 2 * ctx->L + 1];
+    const int *sched = &ctx->h_sched[(size_t)k * 3 * (ctx->L + 1)];
+    int np_k = sched[ctx->L], nu_k = sched[update_block<T> * (ctx->L + 1) + ctx->L];
     if (np_k == 0) break;
     RPBA_KERNEL(ctx, n_panel, k_chol_panel<T><<<np_k, 256, 0, ctx->stream>>>(S, Linv, cv, k));
     RPBA_KERNEL(ctx, n_upd, k_chol_update<T><<<ctx->L + nu_k, 256, 0, ctx->stream>>>(S, Linv, cv, k));

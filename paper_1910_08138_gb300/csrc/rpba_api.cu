@@ -479,17 +479,20 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
   ctx->max_tiles = maxT;
   ctx->ytot = yt;
   // factorisation schedule: for step k the tiles of every sub-block, as
-  // prefix sums (panel: T_l - k - 1 tiles; trailing update: its triangle)
+  // prefix sums (panel: T_l - k - 1 tiles; trailing update: its triangle, in
+  // tiles and in blocks of 2 x 2)
   {
     int steps = std::max(maxT - 1, 1);
-    ctx->h_sched.assign((size_t)steps * 2 * (L + 1), 0);
+    ctx->h_sched.assign((size_t)steps * 3 * (L + 1), 0);
     for (int k = 0; k < steps; k++) {
-      int *pb = &ctx->h_sched[(size_t)k * 2 * (L + 1)];
-      int *ub = pb + (L + 1);
+      int *pb = &ctx->h_sched[(size_t)k * 3 * (L + 1)];
+      int *ub = pb + (L + 1), *bb = ub + (L + 1);
       for (int l = 0; l < L; l++) {
         int rem = std::max(ntiles[l] - k - 1, 0);
         pb[l + 1] = pb[l] + rem;
         ub[l + 1] = ub[l] + rem * (rem + 1) / 2;
+        int rb = (rem + 1) / 2;
+        bb[l + 1] = bb[l] + rb * (rb + 1) / 2;
       }
     }
   }

@@ -379,7 +379,7 @@ struct Ctx {
   // since. sigma0_part: 5 sums per chunk, then per sub-block, then the total
   double *f0_cache = nullptr, *sigma0_part = nullptr;
   bool f0_valid = false;
-  std::vector<int> h_sched;  // per factorisation step: prefix sums of panel and update tiles
+  std::vector<int> h_sched;  // per factorisation step: prefix sums of panel tiles, update tiles and 2 x 2 blocks of these
   int *sched = nullptr;
   double *Linv64 = nullptr;
   float *S32 = nullptr, *Linv32 = nullptr, *ir_r32 = nullptr;
