@@ -8,10 +8,11 @@
 // of different sizes, templated on the arithmetic type T:
 //   k_chol_first   tile (0,0): its inverse factor
 //   step k:
-//   k_chol_panel   one CTA per tile row i > k:  L_ik = A_ik Linv_kk^T
-//   k_chol_update  one CTA per trailing tile (i, j), k < j <= i:
-//                  A_ij -= L_ik L_jk^T; the CTA of tile (k+1, k+1) then
-//                  forms its inverse factor, so the next panel can start
+//   k_chol_panel   one CTA per tile row i > k (FP64: four):  L_ik = A_ik Linv_kk^T
+//   k_chol_update  one CTA per trailing tile (i, j), k < j <= i (FP32: per
+//                  2 x 2 of them): A_ij -= L_ik L_jk^T; the CTA of tile
+//                  (k+1, k+1) then forms its inverse factor, so the next panel
+//                  can start
 // The inverted diagonal tiles Linv_kk turn the panel solve into a GEMM and
 // the diagonal steps of the triangular solves into 32 x 32 matrix-vector
 // products. k_trsv_cluster: forward and backward substitution, one thread
@@ -150,7 +151,7 @@ __device__ __forceinline__ double rcp_ulp(double x) {
 // a coordinate was seen). Bound by the chain of 32 roots and quotients, so a warp
 // takes 8 columns in registers without a barrier, four warps the four column
 // blocks, the other four the inverse: one barrier per 8 columns, a reciprocal per
-// column. Steps of 32 sub-blocks of up to 38 cameras, which this chain decides: 30 us
+// column. Steps of 128 sub-blocks of up to 21 tiles, which this chain decides: 30 us
 // with a column per barrier, 19 us like this.
 // ---------------------------------------------------------------------------
 __device__ bool cta_inverse_factor(const double *C, double *out) {
@@ -320,28 +321,46 @@ __device__ inline void load_tile(T *dst, const T *A, int np, int ti, int tj) {
   }
 }
 
+// Panel: A_ik <- A_ik Linv_kk^T, a CTA per tile or, in FP64, per 8 rows of one: a
+// tile is 16,000 cycles of an SM's FP64 pipes (1024 multiply-adds of a warp, 64
+// cycles each on 4 pipes), on the chain of every step, and few tiles leave most
+// SMs idle. Columns c >= 4 g of the product stop at m = c: Linv is lower
+// triangular. Per step, launch included: two sub-blocks of 5 tiles 14.4 -> 8.4 us, eight
+// of 24 tiles 17 -> 10.8 us.
+template <typename T>
+constexpr int panel_split = sizeof(T) == 8 ? 4 : 1;
 template <typename T>
 __global__ void __launch_bounds__(256) k_chol_panel(T *S, const T *Linv, CholView cv, int k) {
+  constexpr int PS = panel_split<T>, R = CT / PS;
   int loc;
-  int l = sched_find(cv.sched + (size_t)k * 3 * (cv.L + 1), cv.L, blockIdx.x, &loc);
+  int l = sched_find(cv.sched + (size_t)k * 3 * (cv.L + 1), cv.L, blockIdx.x / PS, &loc);
   if (!cv.run[l] || cv.fail[l]) return;
   int np = cv.npad[l];
-  int nt = np / CT;
-  int ti = k + 1 + loc;
-  if (ti >= nt) return;
+  int r0 = (k + 1 + loc) * CT + blockIdx.x % PS * R;
+  if (r0 >= np) return;
   T *A = S + cv.off[l];
-  __shared__ T P[CT * CLD], Q[CT * CLD];
-  load_tile<T>(P, A, np, ti, k);
+  __shared__ T P[R * CLD], Q[CT * CLD];
+  for (int e = threadIdx.x; e < R * CT; e += 256) P[(e / CT) * CLD + e % CT] = A[(size_t)(r0 + e / CT) * np + k * CT + e % CT];
   const T *Li = Linv + cv.linv_off[l] + (size_t)k * CT * CT;
-  for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) Q[(e / CT) * CLD + e % CT] = Li[e];
+  for (int e = threadIdx.x; e < CT * CT; e += 256) Q[(e / CT) * CLD + e % CT] = Li[e];
   __syncthreads();
-  T acc[2][2];
-  tile_nt<T>(P, Q, acc);  // A_ik Linv_kk^T
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  if constexpr (PS == 4) {
+    // a warp per 4 columns; warps w and w + 4 share a pipe: a short one with a long one
+    int w = threadIdx.x >> 5, g = w < 4 ? w : 11 - w;
+    int r = threadIdx.x & 7, c = 4 * g + ((threadIdx.x >> 3) & 3);
+    T t = T(0);
+#pragma unroll 4
+    for (int m = 0; m < 4 * g + 4; m++) t = fma(P[r * CLD + m], Q[c * CLD + m], t);
+    A[(size_t)(r0 + r) * np + k * CT + c] = t;
+  } else {
+    T acc[2][2];
+    tile_nt<T>(P, Q, acc);
+    int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
-  for (int r = 0; r < 2; r++)
+    for (int r = 0; r < 2; r++)
 #pragma unroll
-    for (int c = 0; c < 2; c++) A[(size_t)(ti * CT + ty + 16 * r) * np + k * CT + tx + 16 * c] = acc[r][c];
+      for (int c = 0; c < 2; c++) A[(size_t)(r0 + ty + 16 * r) * np + k * CT + tx + 16 * c] = acc[r][c];
+  }
 }
 
 // Trailing update: a CTA takes B x B tiles (rows and columns k + 1 + B a .., on or
@@ -371,13 +390,19 @@ __global__ void __launch_bounds__(256, 4) k_chol_update(T *S, T *Linv, CholView 
     T *A = S + cv.off[l];
     load_tile<T>(P, A, np, k + 1, k);
     __syncthreads();
-    T acc[2][2];
-    tile_nt<T>(P, P, acc);
+    T acc[2][2] = {};  // rows < 16, columns >= 16 are above the diagonal: not formed
+#pragma unroll 8
+    for (int m = 0; m < CT; m++) {
+      T p0 = P[ty * CLD + m], p1 = P[(ty + 16) * CLD + m], q0 = P[tx * CLD + m], q1 = P[(tx + 16) * CLD + m];
+      acc[0][0] = fma(p0, q0, acc[0][0]);
+      acc[1][0] = fma(p1, q0, acc[1][0]);
+      acc[1][1] = fma(p1, q1, acc[1][1]);
+    }
     __syncthreads();  // every thread is done with P
 #pragma unroll
     for (int r = 0; r < 2; r++)
 #pragma unroll
-      for (int c = 0; c < 2; c++) {
+      for (int c = 0; c <= r; c++) {
         int rr = ty + 16 * r, cc = tx + 16 * c;
         P[rr * CLD + cc] = A[(size_t)((k + 1) * CT + rr) * np + (k + 1) * CT + cc] - acc[r][c];
       }
@@ -1029,7 +1054,7 @@ static rpba_status factor(Ctx *ctx, T *S, T *Linv, CholView cv, int T_max) {
     const int *sched = &ctx->h_sched[(size_t)k * 3 * (ctx->L + 1)];
     int np_k = sched[ctx->L], nu_k = sched[update_block<T> * (ctx->L + 1) + ctx->L];
     if (np_k == 0) break;
-    RPBA_KERNEL(ctx, n_panel, k_chol_panel<T><<<np_k, 256, 0, ctx->stream>>>(S, Linv, cv, k));
+    RPBA_KERNEL(ctx, n_panel, k_chol_panel<T><<<np_k * panel_split<T>, 256, 0, ctx->stream>>>(S, Linv, cv, k));
     RPBA_KERNEL(ctx, n_upd, k_chol_update<T><<<ctx->L + nu_k, 256, 0, ctx->stream>>>(S, Linv, cv, k));
   }
   return RPBA_OK;
