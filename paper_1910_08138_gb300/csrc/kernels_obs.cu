@@ -1774,30 +1774,12 @@ __device__ inline void z_of(const float inv[6], const float B[3 * CD], float Zk[
 //   S_ii = U_ii + lambda diag(U_ii) - sum_k N_XC,k^T Z_k,  U_ii = sum_k w A_C^T W A_C
 // and right-hand side y_i = -sum_k w A_C^T W v + sum_k Z_k^T g_X
 #define CB_THREADS 128
-// one observation k (instance q) of camera i: its terms of U, SZ, gc and yz
-// added to acc when act (the point is active)
-template <typename T, int CD>
-__device__ __forceinline__ void cb_obs_body(const View &v, int i, int k, int q, bool act, const ObsT<T> &ob,
-                                            const T *NXC, const T *Z, const T *gX, const T *Ninv, T *acc);
-
-template <typename T, int CD>
-__device__ __forceinline__ void cb_obs(const View &v, int i, int k, int q, bool act, const T *NXC, const T *Z,
-                                       const T *gX, const T *Ninv, T *acc) {
-  ObsT<T> ob;
-  load_obs<T>(v, k, ob);
-  cb_obs_body<T, CD>(v, i, k, q, act, ob, NXC, Z, gX, Ninv, acc);
-}
-
-// FP32 form: the observation already loaded (from the camera-major streams)
-template <typename T, int CD>
-__device__ __forceinline__ void cb_obs_ob(const View &v, int i, int q, bool act, const ObsT<T> &ob, const T *Ninv,
-                                          const T *gX, T *acc) {
-  cb_obs_body<T, CD>(v, i, 0, q, act, ob, nullptr, nullptr, gX, Ninv, acc);
-}
-
-template <typename T, int CD>
-__device__ __forceinline__ void cb_obs_body(const View &v, int i, int k, int q, bool act, const ObsT<T> &ob,
-                                            const T *NXC, const T *Z, const T *gX, const T *Ninv, T *acc) {
+// one observation (instance q) of camera i: its terms of U, SZ, gc and yz added to
+// acc when act (the point is active)
+template <int CD>
+__device__ __forceinline__ void cb_obs(const View &v, int i, int q, bool act, const ObsT<float> &ob, const float *Ninv,
+                                       const float *gX, float *acc) {
+  using T = float;
   constexpr int NU = CD * (CD + 1) / 2;
   ProjJac<T, CD> pj;
   T z;
@@ -1811,23 +1793,18 @@ __device__ __forceinline__ void cb_obs_body(const View &v, int i, int k, int q, 
   }
   const T *gq = gX + 3 * (size_t)q;
   T Bl[3 * CD], Zl[3 * CD], g3[3] = {gq[0], gq[1], gq[2]};
-  if constexpr (sizeof(T) == sizeof(float)) {  // N_XC and Z in registers
+  // N_XC and Z in registers
 #pragma unroll
-    for (int r = 0; r < 3; r++)
+  for (int r = 0; r < 3; r++)
 #pragma unroll
-      for (int c = 0; c < CD; c++) {
-        T a0 = ob.w * (ob.W[0] * pj.Jx[r] + ob.W[1] * pj.Jx[3 + r]);
-        T a1 = ob.w * (ob.W[1] * pj.Jx[r] + ob.W[2] * pj.Jx[3 + r]);
-        Bl[CD * r + c] = a0 * pj.Jc[c] + a1 * pj.Jc[CD + c];
-      }
-    const float *iv = Ninv + 6 * (size_t)q;
-    float inv[6] = {iv[0], iv[1], iv[2], iv[3], iv[4], iv[5]};
-    z_of<CD>(inv, Bl, Zl);
-  } else {
-    const T *B = NXC + 3 * CD * (size_t)k, *Zk = Z + 3 * CD * (size_t)k;
-#pragma unroll
-    for (int e = 0; e < 3 * CD; e++) { Bl[e] = B[e]; Zl[e] = Zk[e]; }
-  }
+    for (int c = 0; c < CD; c++) {
+      T a0 = ob.w * (ob.W[0] * pj.Jx[r] + ob.W[1] * pj.Jx[3 + r]);
+      T a1 = ob.w * (ob.W[1] * pj.Jx[r] + ob.W[2] * pj.Jx[3 + r]);
+      Bl[CD * r + c] = a0 * pj.Jc[c] + a1 * pj.Jc[CD + c];
+    }
+  const float *iv = Ninv + 6 * (size_t)q;
+  float inv[6] = {iv[0], iv[1], iv[2], iv[3], iv[4], iv[5]};
+  z_of<CD>(inv, Bl, Zl);
   if (!act) return;
   int e = 0;
 #pragma unroll
@@ -1842,10 +1819,10 @@ __device__ __forceinline__ void cb_obs_body(const View &v, int i, int k, int q, 
   }
 }
 
-template <typename T, int CD>
-__global__ void __launch_bounds__(CB_THREADS) k_camera_blocks(View v, const double *lambda, const int *run,
-                                                              const T *NXC, const T *Z, const T *gX,
-                                                              const T *Ninv) {
+template <int CD>
+__global__ void __launch_bounds__(CB_THREADS) k_camera_blocks_f(View v, const double *lambda, const int *run,
+                                                                const float *gX, const float *Ninv) {
+  using T = float;
   constexpr int NU = CD * (CD + 1) / 2;  // upper triangle of a CD x CD block
   constexpr int NA = 2 * NU + 2 * CD;    // U, SZ, gc, yz
   int i = blockIdx.x;
@@ -1857,32 +1834,23 @@ __global__ void __launch_bounds__(CB_THREADS) k_camera_blocks(View v, const doub
 #pragma unroll
   for (int e = 0; e < NA; e++) acc[e] = 0;
   const int p1 = v.cam_obs_ptr[i + 1];
-  if constexpr (sizeof(T) == sizeof(float)) {
-    // the camera's observations from the camera-major streams (coalesced);
-    // only the robust weight (it changes) is gathered by observation, and the
-    // point's active flag is read beside the other gathers, not before them
-    for (int p = v.cam_obs_ptr[i] + threadIdx.x; p < p1; p += CB_THREADS) {
-      int q = v.cm_inst[p];
-      const bool act = v.active[v.cm_pt[p]] != 0;
-      ObsT<float> ob;
-      ob.x = v.cm_xy32[2 * (size_t)p];
-      ob.y = v.cm_xy32[2 * (size_t)p + 1];
-      if (v.has_winv) {
-        ob.W[0] = v.cm_winv32[3 * (size_t)p]; ob.W[1] = v.cm_winv32[3 * (size_t)p + 1];
-        ob.W[2] = v.cm_winv32[3 * (size_t)p + 2];
-      } else {
-        ob.W[0] = 1.f; ob.W[1] = 0.f; ob.W[2] = 1.f;
-      }
-      ob.w = v.obs_w32[v.cam_obs[p]];
-      cb_obs_ob<T, CD>(v, i, q, act, ob, Ninv, gX, acc);
+  // the camera's observations from the camera-major streams (coalesced);
+  // only the robust weight (it changes) is gathered by observation, and the
+  // point's active flag is read beside the other gathers, not before them
+  for (int p = v.cam_obs_ptr[i] + threadIdx.x; p < p1; p += CB_THREADS) {
+    int q = v.cm_inst[p];
+    const bool act = v.active[v.cm_pt[p]] != 0;
+    ObsT<float> ob;
+    ob.x = v.cm_xy32[2 * (size_t)p];
+    ob.y = v.cm_xy32[2 * (size_t)p + 1];
+    if (v.has_winv) {
+      ob.W[0] = v.cm_winv32[3 * (size_t)p]; ob.W[1] = v.cm_winv32[3 * (size_t)p + 1];
+      ob.W[2] = v.cm_winv32[3 * (size_t)p + 2];
+    } else {
+      ob.W[0] = 1.f; ob.W[1] = 0.f; ob.W[2] = 1.f;
     }
-  } else {
-    for (int p = v.cam_obs_ptr[i] + threadIdx.x; p < p1; p += CB_THREADS) {
-      int k = v.cam_obs[p];
-      int q = v.obs_inst[k];
-      if (!v.active[v.inst_pt[q]]) continue;
-      cb_obs<T, CD>(v, i, k, q, true, NXC, Z, gX, Ninv, acc);
-    }
+    ob.w = v.obs_w32[v.cam_obs[p]];
+    cb_obs<CD>(v, i, q, act, ob, Ninv, gX, acc);
   }
   // warp reduction, then across the CTA's warps
   __shared__ T red[CB_THREADS / 32][NA];
@@ -1916,6 +1884,110 @@ __global__ void __launch_bounds__(CB_THREADS) k_camera_blocks(View v, const doub
     double *yv = v.y + v.ycam_off[l];
     for (int r = 0; r < CD; r++) yv[CD * li + r] = -(double)gc[r] + (double)yz[r];
   }
+}
+
+// FP64 form. N_XC = a^T A_C with the two rows a = w W A_X, so N_XC^T Z = A_C^T (a N^-1
+// a^T) A_C: the block is A_C^T (w W - a N^-1 a^T) A_C with a 2 x 2 matrix in the
+// middle, formed in registers; neither N_XC nor Z is read, and U itself is needed on
+// the diagonal only (damping). Bound by FP64 instructions (64 cycles each on a
+// scheduler's pipe): U and N_XC^T Z apart and a shuffle tree per sum took about 530
+// per warp of 32 observations, of which the 54 trees 270; this takes about 200, the 33
+// sums by halving the set that a lane holds at every step of the tree.
+// 1000 cameras, 600,000 observations: 275 -> 245 us; 50 cameras, 8,000: 44 -> 34 us.
+template <int N, int OFF>
+__device__ __forceinline__ void warp_sums_step(double *a, int lane, int base, int cnt, double *out) {
+  if constexpr (OFF == 0) {
+#pragma unroll
+    for (int e = 0; e < N; e++)
+      if (e < cnt) out[base + e] = a[e];
+  } else {
+    constexpr int H = (N + 1) / 2;
+    const bool up = lane & OFF;  // this lane keeps values H .. N - 1
+#pragma unroll
+    for (int e = 0; e < H; e++) {
+      double hi = e + H < N ? a[e + H] : 0.0;
+      double send = up ? a[e] : hi;
+      a[e] = (up ? hi : a[e]) + __shfl_xor_sync(0xffffffffu, send, OFF);
+    }
+    warp_sums_step<H, OFF / 2>(a, lane, base + (up ? H : 0), up ? cnt - H : min(cnt, H), out);
+  }
+}
+
+template <int CD>
+__global__ void __launch_bounds__(CB_THREADS)
+    k_camera_blocks_d(View v, const double *lambda, const int *run, const double *gX, const double *Ninv) {
+  constexpr int NU = CD * (CD + 1) / 2;  // upper triangle of a CD x CD block
+  constexpr int NA = NU + 2 * CD;        // block without damping, diagonal of U, right-hand side
+  int i = blockIdx.x;
+  if (i >= v.M) return;
+  int l = v.cam_sub[i];
+  if (!run[l]) return;
+  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double acc[NA];
+#pragma unroll
+  for (int e = 0; e < NA; e++) acc[e] = 0.0;
+  for (int p = v.cam_obs_ptr[i] + threadIdx.x; p < v.cam_obs_ptr[i + 1]; p += CB_THREADS) {
+    int k = v.cam_obs[p];
+    int q = v.obs_inst[k];
+    if (!v.active[v.inst_pt[q]]) continue;
+    ObsT<double> ob;
+    load_obs<double>(v, k, ob);
+    ProjJac<double, CD> pj;
+    double z;
+    obs_proj<double, CD>(v, i, v.Xl + 3 * (size_t)q, v.Xl_hi + 3 * (size_t)q, v.Xl_lo + 3 * (size_t)q, pj, z);
+    double r0 = pj.u - ob.x, r1 = pj.v - ob.y;
+    double W0 = ob.w * ob.W[0], W1 = ob.w * ob.W[1], W2 = ob.w * ob.W[2];
+    const double *iv = Ninv + 6 * (size_t)q, *gq = gX + 3 * (size_t)q;
+    double a0[3], a1[3], n0[3], n1[3];
+#pragma unroll
+    for (int r = 0; r < 3; r++) {
+      a0[r] = W0 * pj.Jx[r] + W1 * pj.Jx[3 + r];
+      a1[r] = W1 * pj.Jx[r] + W2 * pj.Jx[3 + r];
+    }
+#pragma unroll
+    for (int r = 0; r < 3; r++) {
+      double i0 = iv[s3idx(r, 0)], i1 = iv[s3idx(r, 1)], i2 = iv[s3idx(r, 2)];
+      n0[r] = i0 * a0[0] + i1 * a0[1] + i2 * a0[2];
+      n1[r] = i0 * a1[0] + i1 * a1[1] + i2 * a1[2];
+    }
+    double V0 = W0 - (a0[0] * n0[0] + a0[1] * n0[1] + a0[2] * n0[2]);
+    double V1 = W1 - (a0[0] * n1[0] + a0[1] * n1[1] + a0[2] * n1[2]);
+    double V2 = W2 - (a1[0] * n1[0] + a1[1] * n1[1] + a1[2] * n1[2]);
+    double h0 = n0[0] * gq[0] + n0[1] * gq[1] + n0[2] * gq[2] - (W0 * r0 + W1 * r1);
+    double h1 = n1[0] * gq[0] + n1[1] * gq[1] + n1[2] * gq[2] - (W1 * r0 + W2 * r1);
+    int e = 0;
+#pragma unroll
+    for (int r = 0; r < CD; r++) {
+      double j0 = pj.Jc[r], j1 = pj.Jc[CD + r];
+      double b0 = V0 * j0 + V1 * j1, b1 = V1 * j0 + V2 * j1;
+#pragma unroll
+      for (int c = r; c < CD; c++, e++) acc[e] += b0 * pj.Jc[c] + b1 * pj.Jc[CD + c];
+      acc[NU + r] += j0 * (W0 * j0 + W1 * j1) + j1 * (W1 * j0 + W2 * j1);
+      acc[NU + CD + r] += h0 * j0 + h1 * j1;
+    }
+  }
+  __shared__ double red[CB_THREADS / 32][NA];
+  warp_sums_step<NA, 16>(acc, lane, 0, NA, red[wid]);
+  __syncthreads();
+  if (threadIdx.x < NA) {
+    double x = 0.0;
+    for (int w = 0; w < CB_THREADS / 32; w++) x += red[w][threadIdx.x];
+    red[0][threadIdx.x] = x;
+  }
+  __syncthreads();
+  int e = threadIdx.x, li = v.cam_local[i];
+  if (e < NU) {
+    int r = 0, c = e;
+    while (c >= CD - r) c -= CD - r, r++;
+    c += r;
+    int np = v.npad[l];
+    double *S = v.S + v.S_off[l];
+    double val = red[0][e];
+    if (r == c) val += lambda[l] * red[0][NU + r];
+    S[(size_t)(CD * li + r) * np + CD * li + c] = val;
+    S[(size_t)(CD * li + c) * np + CD * li + r] = val;
+  }
+  if (e < CD) v.y[v.ycam_off[l] + CD * li + e] = red[0][NU + CD + e];
 }
 
 // off-diagonal Schur blocks: one thread per (pair, row r):
@@ -2054,8 +2126,8 @@ static rpba_status build_rcs_cd(Ctx *ctx, const View &v, const double *lambda_de
   if (ctx->opt.precision == 1) {
     RPBA_KERNEL(ctx, "k_linearize_f32", k_linearize<float, CD><<<nblk(ctx->P, ctx->tune.lin), ctx->tune.lin, 0, ctx->stream>>>(
                                         v, lambda_dev, run_dev, nullptr, nullptr, (float *)ctx->Ninv, (float *)ctx->gX));
-    RPBA_KERNEL(ctx, "k_camera_blocks_f32", k_camera_blocks<float, CD><<<ctx->M, CB_THREADS, 0, ctx->stream>>>(
-        v, lambda_dev, run_dev, nullptr, nullptr, (const float *)ctx->gX, (const float *)ctx->Ninv));
+    RPBA_KERNEL(ctx, "k_camera_blocks_f32", k_camera_blocks_f<CD><<<ctx->M, CB_THREADS, 0, ctx->stream>>>(
+        v, lambda_dev, run_dev, (const float *)ctx->gX, (const float *)ctx->Ninv));
     if (ctx->n_pairs)
       RPBA_KERNEL(ctx, "k_schur_seg", k_schur_seg<CD><<<nblk(ctx->n_items, SC_THREADS), SC_THREADS, 0, ctx->stream>>>(
                                           v, run_dev, ctx->n_items, ctx->sitem, ctx->spair_a, ctx->spair_b,
@@ -2065,8 +2137,8 @@ static rpba_status build_rcs_cd(Ctx *ctx, const View &v, const double *lambda_de
     double *NXC = (double *)ctx->NXC, *Z = (double *)ctx->Z;
     RPBA_KERNEL(ctx, "k_linearize_f64", k_linearize<double, CD><<<nblk(ctx->P, ctx->tune.lin), ctx->tune.lin, 0, ctx->stream>>>(v, lambda_dev, run_dev, NXC, Z,
                                                                     (double *)ctx->Ninv, (double *)ctx->gX));
-    RPBA_KERNEL(ctx, "k_camera_blocks_f64", k_camera_blocks<double, CD><<<ctx->M, CB_THREADS, 0, ctx->stream>>>(
-        v, lambda_dev, run_dev, NXC, Z, (const double *)ctx->gX, (const double *)ctx->Ninv));
+    RPBA_KERNEL(ctx, "k_camera_blocks_f64", k_camera_blocks_d<CD><<<ctx->M, CB_THREADS, 0, ctx->stream>>>(
+        v, lambda_dev, run_dev, (const double *)ctx->gX, (const double *)ctx->Ninv));
     if (ctx->n_pairs)
       RPBA_KERNEL(ctx, "k_schur_pairs", k_schur_pairs<double, CD><<<nblk(ctx->n_pairs * CD, 256), 256, 0, ctx->stream>>>(
           v, run_dev, ctx->pair_a, ctx->pair_b, ctx->n_pairs, NXC, Z));
