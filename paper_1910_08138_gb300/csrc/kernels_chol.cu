@@ -136,14 +136,16 @@ __device__ __forceinline__ double rcp_ulp(double x) {
 // step, the rows scaled by D^-1/2 at the end. Thread (row = lane, warp w) holds
 // columns w, w + 8, w + 16, w + 24 of both halves: at step j a column c > j is
 // updated in C, a column c <= j in I, so every step does the same 32 x 32
-// updates. The warp that owns column j + 1 updates it first and publishes it
-// while the others work: one barrier per step. One warp alone gets a quarter of
+// updates. The warp that owns column j + 1 updates it first and publishes it; an
+// mbarrier per column instead of a CTA barrier per step lets it go on to its
+// other columns, and the others to theirs, without waiting for one another.
+// One warp alone gets a quarter of
 // the SM's FP64 rate (each of the four schedulers has its own FP64 pipe, 64
 // cycles per instruction): a tile took 93 us by one warp with a square root and
 // a division per column, 57 us without the divisions, 29 us by eight warps
-// (launch included). Whole factorisations, with the diagonal tiles' CTAs first
-// in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.23 ms, eight of
-// 750 3.2 -> 1.7 ms.
+// and a CTA barrier per step, 24 us without the barriers (launch included). Whole factorisations, with the diagonal tiles' CTAs first
+// in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.17 ms, eight of
+// 750 3.2 -> 1.4 ms (with the panel's split).
 //
 // FP32: square root and division per column, each entry's operations in the
 // order of warp_potrf_inv, so both give the same bits: the refinement of a badly
@@ -154,8 +156,14 @@ __device__ __forceinline__ double rcp_ulp(double x) {
 // column. Steps of 128 sub-blocks of up to 21 tiles, which this chain decides: 30 us
 // with a column per barrier, 19 us like this.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+
 __device__ bool cta_inverse_factor(const double *C, double *out) {
-  __shared__ double lcol[2][CT], dv[CT];
+  __shared__ double Ls[CT][CT], dv[CT];
+  __shared__ __align__(8) uint64_t ready[CT];  // column j of Ls and dv[j] are there
+  __shared__ int late;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double a[4], e[4];
 #pragma unroll
@@ -164,19 +172,25 @@ __device__ bool cta_inverse_factor(const double *C, double *out) {
     a[i] = lane >= c ? C[lane * CLD + c] : C[c * CLD + lane];
     e[i] = lane == c ? 1.0 : 0.0;
   }
+  if (threadIdx.x < CT) tc::mbar_init(&ready[threadIdx.x], 1);
+  if (threadIdx.x == 0) late = 0;
+  __syncthreads();
   auto publish = [&](int j, double aj) {  // column j's multipliers, by its owner warp
     double d = __shfl_sync(0xffffffffu, aj, j);
-    lcol[j & 1][lane] = aj * rcp_ulp(d);
+    Ls[j][lane] = aj * rcp_ulp(d);
     if (lane == 0) dv[j] = d;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ready[j]);
   };
+  bool in_time = true;
   if (w == 0) publish(0, a[0]);
 #pragma unroll
   for (int jb = 0; jb < 4; jb++) {
 #pragma unroll 1
     for (int jw = 0; jw < 8; jw++) {
       const int j = 8 * jb + jw;
-      __syncthreads();
-      const double l = lane > j ? lcol[j & 1][lane] : 0.0;
+      if (in_time) in_time = tc::mbar_wait(&ready[j], 0, 500000000ull);
+      const double l = lane > j ? Ls[j][lane] : 0.0;
       // column j + 1 first, by its owner
       const bool own = j + 1 < CT && w == ((j + 1) & 7);
       if (own) {
@@ -199,10 +213,11 @@ __device__ bool cta_inverse_factor(const double *C, double *out) {
       }
     }
   }
+  if (!in_time) late = 1;
   __syncthreads();
   const double d = dv[lane];
   const bool ok = __all_sync(0xffffffffu, d > 0.0);
-  if (!ok) return false;
+  if (!ok || late) return false;
   const double rs = rsqrt(d);
 #pragma unroll
   for (int i = 0; i < 4; i++) out[lane * CT + w + 8 * i] = e[i] * rs;
