@@ -855,7 +855,7 @@ rpba_status point_obs_setup(Ctx *ctx) {
 // FP32 form, one Gauss-Newton iteration of Eq. bars for one point (the
 // kernel below runs them all in one launch): N_j and g_j over all the point's observations at the
 // current X_j (hi + lo), the FP32 solve with the same checks, FP64
-// re-formation and convergence tests as k_isect_point, the position update
+// re-formation and convergence tests as k_isect_fused_d, the position update
 // in float-float. On convergence the refined weights W^l = N_j - N_j^(l):
 // N_j is also summed in float-float, each instance's part N_j^(l) formed again
 // from its observations, and the difference taken in float-float (the FP32
@@ -1633,7 +1633,7 @@ __device__ __noinline__ void instance_normal_fp64(const View &v, int q, double l
 
 // per instance: N_XX (+ W^l, damped), g_X, Ninv. FP64 form: also per
 // observation N_XC = w A_X^T W A_C and Z = Ninv N_XC (both 3x6 row-major),
-// read by the camera and Schur kernels. The FP32 form stores nothing per
+// read by the Schur and back-substitution kernels. The FP32 form stores nothing per
 // observation: its consumers form those blocks again in registers. FP32
 // form: when the FP32 N_XX has a Frobenius condition number above 1e5, N_XX
 // and g_X are formed again in FP64 and the FP64 inverse is rounded to FP32 (an

@@ -561,7 +561,7 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
   // or per-instance array at a time)
   RPBA_TRY(upload(ctx, &ctx->d_pt_inv, ctx->h_pt_inv.data(), (size_t)N));
   RPBA_TRY(upload(ctx, &ctx->d_inst_canon, ctx->h_inst_canon.data(), (size_t)P));
-  ctx->perm_scratch_n = std::max<size_t>(std::max(3 * (size_t)N, 6 * (size_t)P), COV_ROW_BYTES / sizeof(double) + 1);
+  ctx->perm_scratch_n = std::max<size_t>(6 * (size_t)P, ((size_t)N + 1) * COV_ROW_BYTES / sizeof(double) + 1);
   RPBA_TRY(alloc_n(ctx, &ctx->perm_scratch, ctx->perm_scratch_n));
   RPBA_TRY(upload(ctx, &ctx->pt_inst, pin.data(), (size_t)P));
   RPBA_TRY(upload(ctx, &ctx->inst_pt, inst_pt.data(), (size_t)P));
@@ -1194,8 +1194,9 @@ extern "C" rpba_status rpba_covariance(rpba_ctx *h, const int32_t *ids, int32_t 
     idi[e] = ctx->h_pt_perm[ids[e]];
   }
   // Rows go through the context's staging array, as many at a time as it holds
-  // with their ids behind them: two device allocations and their releases per
-  // call were 150 of its 652 us for 100,000 points (now 505).
+  // with their ids behind them (at least one per point: two halves cost a second
+  // round of copies, 93 -> 121 us for 14,401 points). Two device allocations and
+  // their releases per call were 150 of its 652 us for 100,000 points.
   const int rows = (int)std::min<size_t>(n, ctx->perm_scratch_n * sizeof(double) / COV_ROW_BYTES);
   double *dout = ctx->perm_scratch;
   int *di = reinterpret_cast<int *>(dout + 9 * (size_t)rows);

@@ -228,7 +228,7 @@ struct GraphRec;
 
 struct Tuning {
   int isect = 128;    // k_isect_fused_f: points per CTA
-  int lin = 128;      // k_linearize: instances per CTA
+  int lin = 128;      // k_linearize_f: instances per CTA
   int backsub = 128;  // k_backsub: instances per CTA
   int robust = 256;   // k_robust_weights(_f): observations per CTA
 };
