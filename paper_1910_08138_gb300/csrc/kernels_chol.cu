@@ -138,14 +138,14 @@ __device__ __forceinline__ double rcp_ulp(double x) {
 // updated in C, a column c <= j in I, so every step does the same 32 x 32
 // updates. The warp that owns column j + 1 updates it first and publishes it; an
 // mbarrier per column instead of a CTA barrier per step lets it go on to its
-// other columns, and the others to theirs, without waiting for one another.
-// One warp alone gets a quarter of
-// the SM's FP64 rate (each of the four schedulers has its own FP64 pipe, 64
-// cycles per instruction): a tile took 93 us by one warp with a square root and
-// a division per column, 57 us without the divisions, 29 us by eight warps
-// and a CTA barrier per step, 24 us without the barriers (launch included). Whole factorisations, with the diagonal tiles' CTAs first
-// in the update's grid: two sub-blocks of 150 unknowns 0.53 -> 0.17 ms, eight of
-// 750 3.2 -> 1.4 ms (with the panel's split).
+// other columns, and the others to theirs, without waiting for one another. One
+// warp alone gets a quarter of the SM's FP64 rate (each of the four schedulers
+// has its own FP64 pipe, 64 cycles per instruction). A tile, launch included: 93
+// us by one warp with a square root and a division per column, 57 us without the
+// divisions, 29 us by eight warps and a CTA barrier per step, 24 us without the
+// barriers. Whole factorisations, with the diagonal tiles' CTAs first in the
+// update's grid and the panel split: two sub-blocks of 150 unknowns 0.53 -> 0.17
+// ms, eight of 750 3.2 -> 1.4 ms.
 //
 // FP32: square root and division per column, each entry's operations in the
 // order of warp_potrf_inv, so both give the same bits: the refinement of a badly
