@@ -238,13 +238,18 @@ struct Pow2 {
   __device__ __forceinline__ float mul(float x) const { return a != 0.f ? __fmul_rn(__fmul_rn(x, a), b) : scalbnf(x, e); }
 };
 
-// FP32 form, refinement residual: q += S (X + dx) in float-float over the
+// FP32 form, refinement residual: q = S (X + dx) in float-float over the
 // lower tiles of the active sub-blocks (X float-float, dx the FP32 solution of
-// the stage just ended), summed over the tiles with FP64 atomics. One warp per
-// tile, the warps striding over the tile table (as k_pcg_symv32): lane c reads
-// column c's hi and lo words one row at a time and accumulates the transposed
-// product in float-float; a transposing butterfly of float-float additions over
-// the 32 row terms (hi, lo) leaves row r's sum in lane r.
+// the stage just ended). A tile's parts go to slots of their own, which
+// slot_sum4 adds up whatever the order: the residual is rounded to FP32 for the
+// next stage, so with FP64 atomics their order decided single digits of it and,
+// through the stage, of the solution (one call in ten gave poses and points
+// about 1e-9 away from the others). 10,000 cameras 4.45 -> 4.48 ms per call, 1,000
+// cameras 1.79 ms with both.
+// One warp per tile, the warps striding over the tile table (as k_pcg_symv32):
+// lane c reads column c's hi and lo words one row at a time and accumulates the
+// transposed product in float-float; a transposing butterfly of float-float
+// additions over the 32 row terms (hi, lo) leaves row r's sum in lane r.
 #define SYMV_THREADS 256
 __device__ __forceinline__ float2 warp_transpose_sum_ff(float (&th)[PT / 2], float (&tl)[PT / 2], int lane) {
 #pragma unroll
@@ -264,12 +269,14 @@ __device__ __forceinline__ float2 warp_transpose_sum_ff(float (&th)[PT / 2], flo
 }
 
 // one tile (one warp) at (a, b) of a sub-block: Shi and Slo from its first
-// entry, X, dx and q from its first unknown. HOLD keeps the whole tile in
-// registers between the two products; otherwise (k_pcg_solve, 64 registers) the
-// row terms come from a second pass over the tile, then in the L1.
+// entry, X and dx from its first unknown, part its slots: slot t (np values)
+// takes the part of each unknown that comes from the unknowns of tile row t.
+// HOLD keeps the whole tile in registers between the two products; otherwise
+// (k_pcg_solve, 64 registers) the row terms come from a second pass over the
+// tile, then in the L1.
 template <bool HOLD>
 __device__ __forceinline__ void symv_ff_tile(const float *__restrict__ Shi, const float *__restrict__ Slo, int np,
-                                             int a, int b, const float2 *X, const float *dx, double *q, int lane) {
+                                             int a, int b, const float2 *X, const float *dx, double *part, int lane) {
   const size_t base = (size_t)(a * PT) * np + b * PT + lane;
   Shi += base;
   Slo += base;
@@ -333,18 +340,74 @@ __device__ __forceinline__ void symv_ff_tile(const float *__restrict__ Shi, cons
   }
   float2 row = warp_transpose_sum_ff(th, tl, lane);
   if (!diag) {
-    atomicAdd(q + a * PT + lane, ff_to_double(row));
-    atomicAdd(q + b * PT + lane, ff_to_double(col));
+    part[(size_t)b * np + a * PT + lane] = ff_to_double(row);
+    part[(size_t)a * np + b * PT + lane] = ff_to_double(col);
   } else {
-    atomicAdd(q + a * PT + lane, ff_to_double(ff_add(row, col)));
+    part[(size_t)a * np + a * PT + lane] = ff_to_double(ff_add(row, col));
   }
+}
+
+// offset of a sub-block's slots: np / PT of np values each beside its np x np RCS
+static_assert(PT == RPBA_TILE, "S_off counts np x np entries of PT-row tiles");
+__device__ __forceinline__ size_t slot_off(long long S_off) { return (size_t)(S_off / PT); }
+
+// unknowns e .. e + 3 of q (e a multiple of 4; lane's is e + lane % 4), a warp:
+// the sum of its slots as integers of 2^-55 times the largest term's power of
+// two, so that it is within 2^-56 of that per term (an FP64 addition rounds to
+// 2^-53 of its sum) whatever the order. FP64 additions cost a scheduler 64
+// cycles each: 24 of them for the 750 unknowns of a sub-block took an SM 5 us.
+// Eight lanes share an unknown, so that every slot is read once and at once.
+// Terms that are all tiny, or infinite or NaN: FP64 additions.
+static_assert(RPBA_PCG_FF_MAX_N / PT <= 64, "64 terms below 2^56 in 63 bits, 8 per lane");
+__device__ __forceinline__ double slot_sum4(const double *part, int np, int e, int lane) {
+  const int nt = np / PT;
+  part += e + (lane & 3);
+  double v[8];
+  int top = 0;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    int t = (lane >> 2) + 8 * k;
+    v[k] = t < nt ? __ldcg(part + (size_t)t * np) : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++) top = max(top, (__double2hiint(v[k]) >> 20) & 0x7ff);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  long long s = 0;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    long long b = __double_as_longlong(v[k]);
+    int down = min(top - (int)((b >> 52) & 0x7ff), 60);
+    unsigned long long m = (((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 3;
+    m = (m + ((1ull << down) >> 1)) >> down;
+    s += b < 0 ? -(long long)m : (long long)m;
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  double r = (double)s * __hiloint2double((top - 55) << 20, 0);  // 2^(top - 1023 - 55)
+  if (__any_sync(0xffffffffu, top < 64 || top == 0x7ff)) {
+    double d = 0.0;
+    for (int k = 0; k < 8; k++) d += v[k];
+    for (int o = 4; o < 32; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (top < 64 || top == 0x7ff) r = d;
+  }
+  return r;
+}
+
+// q from the slots, a warp per 4 unknowns
+__global__ void __launch_bounds__(256) k_pcg_slot_sum(const int *npad, const int *voff, const int *act,
+                                                      const long long *S_off, const double *part, double *q) {
+  int l = blockIdx.y, lane = threadIdx.x & 31, e = 32 * blockIdx.x + 4 * (threadIdx.x >> 5);
+  if (!act[l] || e >= npad[l]) return;  // the same for the whole warp
+  double s = slot_sum4(part + slot_off(S_off[l]), npad[l], e, lane);
+  if (lane < 4) q[voff[l] + e + lane] = s;
 }
 
 __global__ void __launch_bounds__(SYMV_THREADS) k_pcg_symv_ff(const float *__restrict__ Shi,
                                                               const float *__restrict__ Slo, const long long *S_off,
                                                               const int *npad, const int *voff, const int *act,
                                                               const int2 *__restrict__ tile_map, int tiles,
-                                                              const float2 *X, const float *dx, double *q) {
+                                                              const float2 *X, const float *dx, double *part) {
   int lane = threadIdx.x & 31;
   int nw = gridDim.x * (SYMV_THREADS / 32);
   for (int idx = blockIdx.x * (SYMV_THREADS / 32) + (threadIdx.x >> 5); idx < tiles; idx += nw) {
@@ -352,7 +415,7 @@ __global__ void __launch_bounds__(SYMV_THREADS) k_pcg_symv_ff(const float *__res
     int l = tm.x;
     if (!act[l]) continue;  // the same for the whole warp
     symv_ff_tile<true>(Shi + S_off[l], Slo + S_off[l], npad[l], tm.y >> 16, tm.y & 0xffff, X + voff[l], dx + voff[l],
-                 q + voff[l], lane);
+                       part + slot_off(S_off[l]), lane);
   }
 }
 
@@ -513,7 +576,7 @@ __device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
 // FP32 form: start of a refinement stage, one CTA per active sub-block.
 // first: X = 0 and R = y (every running sub-block becomes active); otherwise
 // X += x, the FP32 solution of the stage just ended, and R = y - q with
-// q = S X from k_pcg_symv_ff (q is zeroed once read). The solve of the
+// q = S X (qd). The solve of the
 // sub-block ends when ||R|| <= tol ||y||, when a stage has not halved ||R||,
 // after max_stage stages, or at the CG step cap (fin: the device loop's step
 // count loop_cnt[0] at max_iter, or the host loop's last stage);
@@ -524,7 +587,7 @@ __device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
 template <int CD>
 __device__ bool pcg_stage_body(
     int first, bool fin, int l, const int *run, const int *fail, const int *sub_cam_ptr, const int *voff,
-    const int *npad, const float *__restrict__ Minv32, const double *__restrict__ y, double *qd, float2 *X,
+    const int *npad, const float *__restrict__ Minv32, const double *__restrict__ y, const double *qd, float2 *X,
     float *x, float *r, float *z, float *p, unsigned long long *q, double *st, float *s32, int *act, int *live,
     double tol, double tol_in, int max_stage) {
   __shared__ int stop;
@@ -566,7 +629,6 @@ __device__ bool pcg_stage_body(
     } else if (first) {
       X[o + e] = make_float2(0.f, 0.f);
     }
-    qd[o + e] = 0.0;
     r[o + e] = re;
     x[o + e] = 0.f;
     z[o + e] = 0.f;
@@ -634,7 +696,7 @@ template <int CD>
 __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
     int first, int final_stage, const int *loop_cnt, int max_iter, const int *run, const int *fail,
     const int *sub_cam_ptr, const int *voff, const int *npad, const float *__restrict__ Minv32,
-    const double *__restrict__ y, double *qd, float2 *X, float *x, float *r, float *z, float *p,
+    const double *__restrict__ y, const double *qd, float2 *X, float *x, float *r, float *z, float *p,
     unsigned long long *q, double *st, float *s32, int *act, int *live, double tol, double tol_in, int max_stage) {
   pcg_stage_body<CD>(first, final_stage || (loop_cnt && loop_cnt[0] >= max_iter), blockIdx.x, run, fail, sub_cam_ptr, voff, npad, Minv32, y, qd, X, x, r,
                      z, p, q, st, s32, act, live, tol, tol_in, max_stage);
@@ -889,7 +951,7 @@ struct PcgSolve {
   const int2 *tile_map;
   const float *Shi, *Slo, *Minv32;
   const double *y;
-  double *qd;
+  double *part, *qd;
   float2 *X;
   float *x, *r, *z, *p;
   unsigned long long *q;
@@ -917,6 +979,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
   const int np = v.npad[l], o = v.voff[l], t0 = v.tile_ptr[l], nt = v.tile_ptr[l + 1] - t0;
   const int g0 = v.sub_cam_ptr[l], ncam = v.sub_cam_ptr[l + 1] - g0, n = CD * ncam;
   const float *Shi = v.Shi + v.S_off[l], *Slo = v.Slo + v.S_off[l];
+  double *slots = v.part + slot_off(v.S_off[l]);
   float *w = v.s32 + PCG_S32 * l;
   const float smax = w[S32_SMAX];
   auto tell = [&](int go, int sc) {  // to every CTA of the cluster, ordered by the barrier that follows
@@ -971,7 +1034,12 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
     }
     for (int t = warp; t < nt; t += warps) {
       int pos = v.tile_map[t0 + t].y;
-      symv_ff_tile<RES>(Shi, Slo, np, pos >> 16, pos & 0xffff, v.X + o, v.x + o, v.qd + o, lane);
+      symv_ff_tile<RES>(Shi, Slo, np, pos >> 16, pos & 0xffff, v.X + o, v.x + o, slots, lane);
+    }
+    cluster.sync();
+    for (int e = 4 * warp; e < n; e += 4 * warps) {
+      double t = slot_sum4(slots, np, e, lane);
+      if (lane < 4) v.qd[o + e + lane] = t;
     }
     cluster.sync();
     if (vector_part) {
@@ -1405,6 +1473,8 @@ static rpba_status pcg_read_count(Ctx *ctx, const int *flags, int *n_set, int *r
 // read after as many steps as the same stage took in the previous solve,
 // then every 4; the active count after every stage. pcg_max_iter caps the CG
 // steps of all stages together.
+static dim3 slot_sum_grid(const Ctx *ctx) { return dim3(ctx->max_tiles, ctx->L); }  // 32 unknowns per CTA
+
 static rpba_status pcg_loop_refined(Ctx *ctx, int *iters) {
   int L = ctx->L;
   cudaStream_t st = ctx->stream;
@@ -1439,7 +1509,10 @@ static rpba_status pcg_loop_refined(Ctx *ctx, int *iters) {
     RPBA_KERNEL(ctx, "k_pcg_symv_ff", k_pcg_symv_ff<<<symv32_grid(tiles), SYMV_THREADS, 0, st>>>(
                                           ctx->pcg_Shi, ctx->pcg_Slo, ctx->S_off, ctx->npad, ctx->ycam_off,
                                           ctx->pcg_act, ctx->pcg_tile_map, tiles, ctx->pcg_fx, ctx->pcg_x32,
-                                          ctx->pcg_q));
+                                          ctx->pcg_part));
+    RPBA_KERNEL(ctx, "k_pcg_slot_sum", k_pcg_slot_sum<<<slot_sum_grid(ctx), 256, 0, st>>>(
+                                           ctx->npad, ctx->ycam_off, ctx->pcg_act, ctx->S_off, ctx->pcg_part,
+                                           ctx->pcg_q));
     RPBA_KERNEL(ctx, "k_pcg_stage", stage_k<<<L, PCG_THREADS, 0, st>>>(
                                         0, last ? 1 : 0, nullptr, 0, nullptr, nullptr, ctx->sub_cam_ptr, ctx->ycam_off,
                                         ctx->npad, ctx->pcg_Minv32, ctx->y, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32,
@@ -1474,7 +1547,7 @@ __global__ void __launch_bounds__(256) k_pcg_cond(cudaGraphConditionalHandle h, 
 // the phases of k_pcg_solve as the profile lists them: the names of the kernels
 // that run them when launched one by one
 static const char *const kCgPhases[] = {"k_pcg_symv32", "k_pcg_step32", "k_pcg_cond"};
-static const char *const kStagePhases[] = {"k_pcg_symv_ff", "k_pcg_stage", "k_pcg_cond"};
+static const char *const kStagePhases[] = {"k_pcg_symv_ff", "k_pcg_slot_sum", "k_pcg_stage", "k_pcg_cond"};
 
 static bool pcg_loop_kernel(const std::string &n) {
   for (const char *k : kCgPhases)
@@ -1607,7 +1680,10 @@ static rpba_status pcg_loop_device(Ctx *ctx) {
     RPBA_KERNEL(ctx, "k_pcg_symv_ff", k_pcg_symv_ff<<<symv32_grid(tiles), SYMV_THREADS, 0, bo>>>(
                                           ctx->pcg_Shi, ctx->pcg_Slo, ctx->S_off, ctx->npad, ctx->ycam_off,
                                           ctx->pcg_act, ctx->pcg_tile_map, tiles, ctx->pcg_fx, ctx->pcg_x32,
-                                          ctx->pcg_q));
+                                          ctx->pcg_part));
+    RPBA_KERNEL(ctx, "k_pcg_slot_sum", k_pcg_slot_sum<<<slot_sum_grid(ctx), 256, 0, bo>>>(
+                                           ctx->npad, ctx->ycam_off, ctx->pcg_act, ctx->S_off, ctx->pcg_part,
+                                           ctx->pcg_q));
     RPBA_KERNEL(ctx, "k_pcg_stage", stage_k<<<L, PCG_THREADS, 0, bo>>>(
                                         0, 0, cnt, maxit, nullptr, nullptr, ctx->sub_cam_ptr, ctx->ycam_off,
                                         ctx->npad, ctx->pcg_Minv32, ctx->y, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32,
@@ -1670,8 +1746,8 @@ static rpba_status pcg_solve(Ctx *ctx, int *iters) {
   RPBA_CUDA(cudaMemsetAsync(cnt, 0, cnt_bytes, st));
   PcgSolve v{ctx->opt.pcg_max_iter, RPBA_PCG_MAX_STAGES, ctx->pcg_minv_smem, ctx->sub_cam_ptr, ctx->ycam_off,
              ctx->npad, ctx->pcg_tiles, ctx->S_off, ctx->pcg_tile_map, ctx->pcg_Shi, ctx->pcg_Slo, ctx->pcg_Minv32,
-             ctx->y, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32, ctx->pcg_r32, ctx->pcg_z32, ctx->pcg_p32, ctx->pcg_qi,
-             ctx->pcg_st, ctx->pcg_s32, ctx->pcg_act, ctx->pcg_live, cnt, ctx->opt.pcg_tol, RPBA_PCG_INNER_TOL};
+             ctx->y, ctx->pcg_part, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32, ctx->pcg_r32, ctx->pcg_z32, ctx->pcg_p32,
+             ctx->pcg_qi, ctx->pcg_st, ctx->pcg_s32, ctx->pcg_act, ctx->pcg_live, cnt, ctx->opt.pcg_tol, RPBA_PCG_INNER_TOL};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctx->pcg_cluster * ctx->L);
   cfg.blockDim = dim3(ctx->pcg_res ? 8 * 32 : 32 * 32);

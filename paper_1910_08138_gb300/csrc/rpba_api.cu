@@ -725,6 +725,7 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
       RPBA_TRY(pcg_solve_setup(ctx, max_n));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_Shi, (size_t)std::max(stot, 1LL)));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_Slo, (size_t)std::max(stot, 1LL)));
+      RPBA_TRY(alloc_n(ctx, &ctx->pcg_part, (size_t)std::max(stot / RPBA_TILE, 1LL)));
       RPBA_TRY(alloc_n(ctx, &ctx->pcg_fx, (size_t)std::max(yt, 1)));
       for (float **v : {&ctx->pcg_x32, &ctx->pcg_r32, &ctx->pcg_z32, &ctx->pcg_p32})
         RPBA_TRY(alloc_n(ctx, v, (size_t)std::max(yt, 1)));

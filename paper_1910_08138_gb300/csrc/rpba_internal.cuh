@@ -323,6 +323,7 @@ struct Ctx {
   float2 *pcg_fx = nullptr;
   float *pcg_x32 = nullptr, *pcg_r32 = nullptr, *pcg_z32 = nullptr, *pcg_p32 = nullptr;
   unsigned long long *pcg_qi = nullptr;  // the CG product S_hi p in 64-bit fixed point
+  double *pcg_part = nullptr;             // the residual's product by tile, slots of a sub-block at S_off / 32
   int2 *pcg_tile_map = nullptr;           // per lower tile of the running RCS: (sub-block, a << 16 | b)
   float *pcg_Minv32 = nullptr, *pcg_s32 = nullptr;
   int *pcg_act = nullptr;
