@@ -12,7 +12,7 @@
 // current, through cudaGetSymbolAddress (first call on the device), and passes
 // that address to the kernels. Every call shares the array and it keeps the
 // previous call's contents; each block overwrites its own slots before they are
-// read, and the count of arrivals restarts with each call's number. Calls whose work
+// read, and a call leaves its count of arrivals at zero. Calls whose work
 // overlaps on the GPU (two streams, or two host threads) race on the array.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -29,19 +29,18 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kObsBlocks = RPBA_NOALLOC_MAX_OBS / kThreads;
 constexpr int kPtBlocks = RPBA_NOALLOC_MAX_POINTS / kThreads;
-// layout: 4 doubles per observation block, 1 per point block, 5 final sums, and
-// the word that counts arrivals
-constexpr int kArrived = 4 * kObsBlocks + kPtBlocks + 5;
-constexpr int kSlots = kArrived + 3;
-constexpr int kCountBits = 20;  // CTAs of one call
-static_assert(kObsBlocks + kPtBlocks < 1 << kCountBits, "arrivals of one call");
+// layout: 4 doubles per observation block, 1 per point block, 5 final sums (and
+// 3 unused), and the words that count arrivals
+constexpr int kArrived = 4 * kObsBlocks + kPtBlocks + 8;
+constexpr int kCounters = 1024;
+constexpr int kSlots = kArrived + kCounters / 2;
 
 static __device__ __align__(256) double g_scratch[kSlots];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 double *g_scratch_dev[kMaxDevices] = {nullptr};
-std::atomic<unsigned long long> g_calls{0};
+std::atomic<unsigned> g_calls{0};
 
 __device__ inline void block_sum(double *v, int nv, double *out) {
   __shared__ double sh[8][kThreads / 32];
@@ -67,14 +66,14 @@ __device__ inline void block_sum(double *v, int nv, double *out) {
 // 47.1 us per call at 8000 observations, this one takes 43.6 us (call, copy
 // back and synchronisation included).
 //
-// Arrival is counted in one word that holds the call's number above the count:
-// the first arrival of a call raises it to (call, 0). A count left over by calls
-// that overlapped is thus never seen by a later call.
+// Arrivals are counted from zero to the call's last, who sets the word back, so
+// calls whose work does not overlap need no order among them. Successive calls
+// take successive words of a ring: as many calls as the ring has words can
+// overlap (and race on the sums) without a count that a later call would meet.
 __global__ void __launch_bounds__(kThreads)
     k_na_sigma0(int K, int N, int n_obs_blocks, const double *R, const double *t, const double *intr, const double *X,
                 const uint8_t *active, const int32_t *obs_cam, const int32_t *obs_point, const double *obs_xy,
-                const double *obs_winv, const double *obs_w, unsigned long long call, unsigned long long *arrived,
-                double *scratch) {
+                const double *obs_winv, const double *obs_w, unsigned *arrived, double *scratch) {
   if ((int)blockIdx.x < n_obs_blocks) {
     int k = blockIdx.x * kThreads + threadIdx.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -108,10 +107,7 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ int last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (__ldcg(arrived) >> kCountBits < call) atomicMax(arrived, call << kCountBits);
-    last = atomicAdd(arrived, 1ull) + 1 == (call << kCountBits) + gridDim.x;
-  }
+  if (threadIdx.x == 0) last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;  // the last one's wraps to zero
   __syncthreads();
   if (!last) return;
   __threadfence();
@@ -157,9 +153,9 @@ extern "C" rpba_status rpba_sigma0_noalloc(int32_t n_cams, int32_t n_points, int
   cudaStream_t s = (cudaStream_t)cuda_stream;
   int nbo = (n_obs + kThreads - 1) / kThreads, nbp = (n_points + kThreads - 1) / kThreads;
   nbp = std::max(nbp, nbo ? 0 : 1);  // an empty block: one CTA writes its zero sums
+  unsigned *arrived = reinterpret_cast<unsigned *>(scratch + kArrived) + g_calls++ % kCounters;
   k_na_sigma0<<<nbo + nbp, kThreads, 0, s>>>(n_obs, n_points, nbo, R, t, intr, X, active, obs_cam, obs_point, obs_xy,
-                                             obs_winv, obs_w, ++g_calls, (unsigned long long *)(scratch + kArrived),
-                                             scratch);
+                                             obs_winv, obs_w, arrived, scratch);
   if (cudaGetLastError() != cudaSuccess) return RPBA_ERR_CUDA;
   double h[5];
   if (cudaMemcpyAsync(h, scratch + 4 * (size_t)kObsBlocks + kPtBlocks, sizeof(h), cudaMemcpyDeviceToHost, s) !=
