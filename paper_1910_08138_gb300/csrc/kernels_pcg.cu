@@ -574,9 +574,9 @@ __device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
 }
 
 // FP32 form: start of a refinement stage, one CTA per active sub-block.
-// first: X = 0 and R = y (every running sub-block becomes active); otherwise
-// X += x, the FP32 solution of the stage just ended, and R = y - q with
-// q = S X (qd). The solve of the
+// first: X = 0 and R = y (every running sub-block becomes active, or this one
+// when run is null); otherwise X += x, the FP32 solution of the stage just
+// ended, and R = y - q with q = S X (qd). The solve of the
 // sub-block ends when ||R|| <= tol ||y||, when a stage has not halved ||R||,
 // after max_stage stages, or at the CG step cap (fin: the device loop's step
 // count loop_cnt[0] at max_iter, or the host loop's last stage);
@@ -593,7 +593,7 @@ __device__ bool pcg_stage_body(
   __shared__ int stop;
   int stage;
   if (first) {
-    int ok = run[l] && !fail[l];
+    int ok = !run || (run[l] && !fail[l]);
     if (threadIdx.x == 0) {
       act[l] = ok;
       live[l] = 0;
@@ -944,6 +944,14 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
 // 1,000-camera call 1.89 -> 1.79 ms).
 // stage_steps: per stage the most CG steps any sub-block took (max_stage
 // entries), then the most stages.
+// max_iter caps the steps of a solve whose sub-blocks go through the stages
+// together: the sum of the stages' counts, which no cluster knows while it
+// runs. A second launch (REDO) therefore looks whether the sum reached the cap,
+// returns if not (2 us), and otherwise solves the sub-blocks that got into the
+// stage where it did once more, with what the stages before left of the cap for
+// that stage and none after it. (The same behind the solve in this kernel cost
+// its loop's code 6 us per LM step of two sub-blocks of 150 unknowns, a
+// conditional loop of the single kernels 12 us.)
 struct PcgSolve {
   int max_iter, max_stage, minv_in_smem;
   const int *sub_cam_ptr, *voff, *npad, *tile_ptr;
@@ -965,15 +973,23 @@ struct PcgSolve {
 // the whole solve. Else the tiles come from the L2 or memory every step, and
 // 32 warps per CTA hide a tile's chain (position, entries, p, butterfly: about
 // 3,000 cycles of latency for 300 instructions).
-template <int CD, int WARPS, bool RES>
+template <int CD, int WARPS, bool RES, bool REDO>
 __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
   namespace cg = cooperative_groups;
+  int last = RPBA_PCG_MAX_STAGES, budget = 0;  // REDO: the stage that reaches the cap, and its steps
+  if constexpr (REDO) {
+    int sum = 0;
+    for (int k = 0; k < RPBA_PCG_MAX_STAGES; k++) sum += v.stage_steps[k];
+    if (sum < v.max_iter) return;
+    while (sum >= v.max_iter) sum -= v.stage_steps[--last];
+    budget = v.max_iter - sum;
+  }
   extern __shared__ __align__(16) float vec[];  // CTA 0: x, r, z, p and M^-1 (when it fits) of the sub-block
   __shared__ int ctl[2];  // CTA 0's decision: go on; the exponent of the next product
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
   const int l = blockIdx.x / C;
-  if (!v.act[l]) return;  // uniform over the cluster
+  if (REDO ? (int)v.s32[PCG_S32 * l + S32_STAGES] <= last : !v.act[l]) return;  // uniform over the cluster
   const int lane = threadIdx.x & 31, warp = rank * WARPS + (threadIdx.x >> 5), warps = C * WARPS;
   const bool vector_part = rank == 0 && threadIdx.x < PCG_THREADS;
   const int np = v.npad[l], o = v.voff[l], t0 = v.tile_ptr[l], nt = v.tile_ptr[l + 1] - t0;
@@ -999,7 +1015,19 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
       symv32_load(Shi, np, ab >> 16, ab & 0xffff, lane, mine);
     }
   }
-  int go = v.live[l], sc = (int)w[S32_QEXP], steps = 0, stages = 0;
+  if constexpr (REDO) {
+    cluster.sync();  // every CTA has read the word that the start resets
+    if (vector_part) {
+      bool more = pcg_stage_body<CD>(1, false, l, nullptr, nullptr, v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y, v.qd,
+                                     v.X, v.x, v.r, v.z, v.p, v.q, v.st, v.s32, v.act, v.live, v.tol, v.tol_in,
+                                     v.max_stage);
+      step_sync();  // thread 0's words of w
+      tell(more, (int)w[S32_QEXP]);
+    }
+    cluster.sync();
+  }
+  int go = REDO ? ctl[0] : v.live[l], sc = REDO ? ctl[1] : (int)w[S32_QEXP];
+  int steps = 0, ran = 0, stages = 0;  // ran: steps without those that broke down
   while (go) {
     CgState s = cg_load(w);
     int in_stage = 0;
@@ -1022,8 +1050,9 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
       cluster.sync();
       if (vector_part) {
         int res = cg_step_body<CD>(ncam, np, smax, minv, v.q + o, v.p + o, vec, s);
-        in_stage += res != 0;
-        const bool more = res == 2 && steps + in_stage < v.max_iter;
+        in_stage++;
+        ran += res != 0;
+        const bool more = res == 2 && in_stage < (REDO && stages == last ? budget : v.max_iter - steps);
         if (!more)  // the stage's solution, for the float-float product
           for (int e = threadIdx.x; e < n; e += PCG_THREADS) v.x[o + e] = vec[e];
         tell(more, s.sc);
@@ -1045,13 +1074,15 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
     if (vector_part) {
       steps += in_stage;
       if (threadIdx.x == 0) {
-        v.st[4 * l + 3] = (double)steps;
-        atomicMax(v.stage_steps + stages, in_stage);
-        atomicMax(v.stage_steps + v.max_stage, stages + 1);
+        v.st[4 * l + 3] = (double)ran;
+        if constexpr (!REDO) {
+          atomicMax(v.stage_steps + stages, in_stage);
+          atomicMax(v.stage_steps + v.max_stage, stages + 1);
+        }
       }
-      bool more = pcg_stage_body<CD>(0, steps >= v.max_iter, l, nullptr, nullptr, v.sub_cam_ptr, v.voff, v.npad,
-                                     v.Minv32, v.y, v.qd, v.X, v.x, v.r, v.z, v.p, v.q, v.st, v.s32, v.act, v.live,
-                                     v.tol, v.tol_in, v.max_stage);
+      bool more = pcg_stage_body<CD>(0, (REDO && stages == last) || steps >= v.max_iter, l, nullptr, nullptr,
+                                     v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y, v.qd, v.X, v.x, v.r, v.z, v.p, v.q,
+                                     v.st, v.s32, v.act, v.live, v.tol, v.tol_in, v.max_stage);
       step_sync();  // thread 0's words of w
       tell(more, (int)w[S32_QEXP]);
     }
@@ -1575,8 +1606,9 @@ int pcg_loop_steps(const Ctx *ctx, int *stages) {
     if (stages) *stages = c[1];
     return c[0];
   }
-  for (int k = 0; k < RPBA_PCG_MAX_STAGES; k++) n += c[k];
-  if (stages) *stages = c[RPBA_PCG_MAX_STAGES];
+  int ran = 0;
+  while (ran < c[RPBA_PCG_MAX_STAGES] && n < ctx->opt.pcg_max_iter) n += c[ran++];  // none after the cap
+  if (stages) *stages = ran;
   return std::min(n, ctx->opt.pcg_max_iter);
 }
 
@@ -1700,9 +1732,10 @@ static rpba_status pcg_loop_device(Ctx *ctx) {
 }
 
 typedef void (*PcgSolveKernel)(PcgSolve);
+template <bool REDO>
 static PcgSolveKernel pcg_solve_kernel(const Ctx *ctx) {
-  if (ctx->cd == 8) return ctx->pcg_res ? k_pcg_solve<8, 8, true> : k_pcg_solve<8, 32, false>;
-  return ctx->pcg_res ? k_pcg_solve<6, 8, true> : k_pcg_solve<6, 32, false>;
+  if (ctx->cd == 8) return ctx->pcg_res ? k_pcg_solve<8, 8, true, REDO> : k_pcg_solve<8, 32, false, REDO>;
+  return ctx->pcg_res ? k_pcg_solve<6, 8, true, REDO> : k_pcg_solve<6, 32, false, REDO>;
 }
 
 // k_pcg_solve or the loop of graph nodes: the nodes spread the products over
@@ -1759,15 +1792,18 @@ static rpba_status pcg_solve(Ctx *ctx, int *iters) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (ctx->L) RPBA_KERNEL(ctx, "k_pcg_solve", RPBA_CUDA(cudaLaunchKernelEx(&cfg, pcg_solve_kernel(ctx), v)));
+  if (ctx->L) RPBA_KERNEL(ctx, "k_pcg_solve", RPBA_CUDA(cudaLaunchKernelEx(&cfg, pcg_solve_kernel<false>(ctx), v)));
+  if (ctx->L > 1)  // one sub-block counts for itself
+    RPBA_KERNEL(ctx, "k_pcg_solve_capped", RPBA_CUDA(cudaLaunchKernelEx(&cfg, pcg_solve_kernel<true>(ctx), v)));
   RPBA_CUDA(cudaMemcpyAsync(ctx->h_pinned_counter + PCG_LOOP_COUNTERS, cnt, cnt_bytes, cudaMemcpyDeviceToHost, st));
   if (iters) *iters = 0;  // in a graph: known after the replay (pinned counters)
   if (ctx->capture) {
     ctx->capture->pcg_loop = true;
     return RPBA_OK;
   }
-  RPBA_CUDA(cudaStreamSynchronize(st));
-  if (iters) *iters = pcg_loop_steps(ctx, nullptr);
+  int n_act, ran;
+  RPBA_TRY(pcg_read_count(ctx, ctx->pcg_act, &n_act, &ran));  // synchronises
+  if (iters) *iters = ran;  // of the slowest sub-block, as the host-driven loop counts them
   pcg_loop_account(ctx, nullptr);
   return RPBA_OK;
 }
