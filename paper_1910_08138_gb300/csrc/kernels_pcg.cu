@@ -359,6 +359,17 @@ __device__ __forceinline__ size_t slot_off(long long S_off) { return (size_t)(S_
 // Eight lanes share an unknown, so that every slot is read once and at once.
 // Terms that are all tiny, or infinite or NaN: FP64 additions.
 static_assert(RPBA_PCG_FF_MAX_N / PT <= 64, "64 terms below 2^56 in 63 bits, 8 per lane");
+__device__ __forceinline__ int slot_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ long long slot_fixed(double v, int top) {
+  long long b = __double_as_longlong(v);
+  int down = min(top - slot_exp(v), 60);
+  unsigned long long m = (((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 3;
+  m = (m + ((1ull << down) >> 1)) >> down;
+  return b < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ double slot_value(long long s, int top) {
+  return (double)s * __hiloint2double((top - 55) << 20, 0);  // 2^(top - 1023 - 55)
+}
 __device__ __forceinline__ double slot_sum4(const double *part, int np, int e, int lane) {
   const int nt = np / PT;
   part += e + (lane & 3);
@@ -370,21 +381,15 @@ __device__ __forceinline__ double slot_sum4(const double *part, int np, int e, i
     v[k] = t < nt ? __ldcg(part + (size_t)t * np) : 0.0;
   }
 #pragma unroll
-  for (int k = 0; k < 8; k++) top = max(top, (__double2hiint(v[k]) >> 20) & 0x7ff);
+  for (int k = 0; k < 8; k++) top = max(top, slot_exp(v[k]));
 #pragma unroll
   for (int o = 4; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
   long long s = 0;
 #pragma unroll
-  for (int k = 0; k < 8; k++) {
-    long long b = __double_as_longlong(v[k]);
-    int down = min(top - (int)((b >> 52) & 0x7ff), 60);
-    unsigned long long m = (((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << 3;
-    m = (m + ((1ull << down) >> 1)) >> down;
-    s += b < 0 ? -(long long)m : (long long)m;
-  }
+  for (int k = 0; k < 8; k++) s += slot_fixed(v[k], top);
 #pragma unroll
   for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  double r = (double)s * __hiloint2double((top - 55) << 20, 0);  // 2^(top - 1023 - 55)
+  double r = slot_value(s, top);
   if (__any_sync(0xffffffffu, top < 64 || top == 0x7ff)) {
     double d = 0.0;
     for (int k = 0; k < 8; k++) d += v[k];
@@ -392,6 +397,25 @@ __device__ __forceinline__ double slot_sum4(const double *part, int np, int e, i
     if (top < 64 || top == 0x7ff) r = d;
   }
   return r;
+}
+
+// the same by one thread, of up to NT terms
+template <int NT>
+__device__ __forceinline__ double slot_sum1(const double *part, int np, int e) {
+  const int nt = np / PT;
+  double v[NT];
+#pragma unroll
+  for (int t = 0; t < NT; t++) v[t] = t < nt ? __ldcg(part + (size_t)t * np + e) : 0.0;
+  int top = 0;
+#pragma unroll
+  for (int t = 0; t < NT; t++) top = max(top, slot_exp(v[t]));
+  long long s = 0;
+  double d = 0.0;
+#pragma unroll
+  for (int t = 0; t < NT; t++) s += slot_fixed(v[t], top);
+  if (top >= 64 && top < 0x7ff) return slot_value(s, top);
+  for (int t = 0; t < NT; t++) d += v[t];
+  return d;
 }
 
 // q from the slots, a warp per 4 unknowns
@@ -576,7 +600,7 @@ __device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
 // FP32 form: start of a refinement stage, one CTA per active sub-block.
 // first: X = 0 and R = y (every running sub-block becomes active, or this one
 // when run is null); otherwise X += x, the FP32 solution of the stage just
-// ended, and R = y - q with q = S X (qd). The solve of the
+// ended, and R = y - q with q = S X (its unknown e: q_of(e)). The solve of the
 // sub-block ends when ||R|| <= tol ||y||, when a stage has not halved ||R||,
 // after max_stage stages, or at the CG step cap (fin: the device loop's step
 // count loop_cnt[0] at max_iter, or the host loop's last stage);
@@ -584,10 +608,10 @@ __device__ __forceinline__ void stage_sum2(double (&v)[2], double (&out)[2]) {
 // z = M^-1 r, p = z, stopping at ||r|| <= max(tol_in, 0.3 tol ||y|| / ||R||)
 // ||R||. st[4l + 2] is the relative true residual ||R|| / ||y||.
 // Returns (uniformly) whether the CG restarts.
-template <int CD>
+template <int CD, class Q>
 __device__ bool pcg_stage_body(
-    int first, bool fin, int l, const int *run, const int *fail, const int *sub_cam_ptr, const int *voff,
-    const int *npad, const float *__restrict__ Minv32, const double *__restrict__ y, const double *qd, float2 *X,
+    Q q_of, int first, bool fin, int l, const int *run, const int *fail, const int *sub_cam_ptr, const int *voff,
+    const int *npad, const float *__restrict__ Minv32, const double *__restrict__ y, float2 *X,
     float *x, float *r, float *z, float *p, unsigned long long *q, double *st, float *s32, int *act, int *live,
     double tol, double tol_in, int max_stage) {
   __shared__ int stop;
@@ -621,7 +645,7 @@ __device__ bool pcg_stage_body(
         v[1] += y[o + e] * y[o + e];
       } else {
         X[o + e] = ff_add(X[o + e], make_float2(x[o + e], 0.f));
-        float2 qf = ff_split_bits(__ldcg(qd + o + e));
+        float2 qf = ff_split_bits(q_of(e));
         R = ff_add(yf, make_float2(-qf.x, -qf.y));
       }
       rr = __fmaf_rn(R.x, R.x, rr);
@@ -698,8 +722,10 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_stage(
     const int *sub_cam_ptr, const int *voff, const int *npad, const float *__restrict__ Minv32,
     const double *__restrict__ y, const double *qd, float2 *X, float *x, float *r, float *z, float *p,
     unsigned long long *q, double *st, float *s32, int *act, int *live, double tol, double tol_in, int max_stage) {
-  pcg_stage_body<CD>(first, final_stage || (loop_cnt && loop_cnt[0] >= max_iter), blockIdx.x, run, fail, sub_cam_ptr, voff, npad, Minv32, y, qd, X, x, r,
-                     z, p, q, st, s32, act, live, tol, tol_in, max_stage);
+  const double *ql = qd + voff[blockIdx.x];
+  pcg_stage_body<CD>([&](int e) { return ql[e]; }, first, final_stage || (loop_cnt && loop_cnt[0] >= max_iter),
+                     blockIdx.x, run, fail, sub_cam_ptr, voff, npad, Minv32, y, X, x, r, z, p, q, st, s32, act, live, tol,
+                     tol_in, max_stage);
 }
 
 // FP32 form, inner CG step of a refinement stage (one CTA per live
@@ -1005,6 +1031,10 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
       c[1] = sc;
     }
   };
+  auto q_of = [&](int e) {
+    if constexpr (RES) return slot_sum1<10>(slots, np, e);  // at most 64 tiles: 10 rows
+    else return __ldcg(v.qd + o + e);
+  };
   const float *minv = v.Minv32 + CD * CD * (size_t)g0;
   if (vector_part && v.minv_in_smem) minv = cg_load_minv<CD>(n, minv, vec);
   float mine[RES ? PT : 1];  // this warp's tile, its lane's column
@@ -1018,7 +1048,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
   if constexpr (REDO) {
     cluster.sync();  // every CTA has read the word that the start resets
     if (vector_part) {
-      bool more = pcg_stage_body<CD>(1, false, l, nullptr, nullptr, v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y, v.qd,
+      bool more = pcg_stage_body<CD>(q_of, 1, false, l, nullptr, nullptr, v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y,
                                      v.X, v.x, v.r, v.z, v.p, v.q, v.st, v.s32, v.act, v.live, v.tol, v.tol_in,
                                      v.max_stage);
       step_sync();  // thread 0's words of w
@@ -1066,11 +1096,13 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
       symv_ff_tile<RES>(Shi, Slo, np, pos >> 16, pos & 0xffff, v.X + o, v.x + o, slots, lane);
     }
     cluster.sync();
-    for (int e = 4 * warp; e < n; e += 4 * warps) {
-      double t = slot_sum4(slots, np, e, lane);
-      if (lane < 4) v.qd[o + e + lane] = t;
+    if constexpr (!RES) {  // else the few terms of an unknown are added where they are read
+      for (int e = 4 * warp; e < n; e += 4 * warps) {
+        double t = slot_sum4(slots, np, e, lane);
+        if (lane < 4) v.qd[o + e + lane] = t;
+      }
+      cluster.sync();
     }
-    cluster.sync();
     if (vector_part) {
       steps += in_stage;
       if (threadIdx.x == 0) {
@@ -1080,9 +1112,9 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
           atomicMax(v.stage_steps + v.max_stage, stages + 1);
         }
       }
-      bool more = pcg_stage_body<CD>(0, (REDO && stages == last) || steps >= v.max_iter, l, nullptr, nullptr,
-                                     v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y, v.qd, v.X, v.x, v.r, v.z, v.p, v.q,
-                                     v.st, v.s32, v.act, v.live, v.tol, v.tol_in, v.max_stage);
+      bool more = pcg_stage_body<CD>(q_of, 0, (REDO && stages == last) || steps >= v.max_iter, l, nullptr, nullptr,
+                                     v.sub_cam_ptr, v.voff, v.npad, v.Minv32, v.y, v.X, v.x, v.r, v.z, v.p, v.q, v.st,
+                                     v.s32, v.act, v.live, v.tol, v.tol_in, v.max_stage);
       step_sync();  // thread 0's words of w
       tell(more, (int)w[S32_QEXP]);
     }
