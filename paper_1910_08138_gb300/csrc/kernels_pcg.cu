@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(PCG_THREADS) k_pcg_step32(const int *sub_cam_p
 // its loop's code 6 us per LM step of two sub-blocks of 150 unknowns, a
 // conditional loop of the single kernels 12 us.)
 struct PcgSolve {
-  int max_iter, max_stage, minv_in_smem;
+  int max_iter, max_stage;
   const int *sub_cam_ptr, *voff, *npad, *tile_ptr;
   const long long *S_off;
   const int2 *tile_map;
@@ -1010,7 +1010,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
     while (sum >= v.max_iter) sum -= v.stage_steps[--last];
     budget = v.max_iter - sum;
   }
-  extern __shared__ __align__(16) float vec[];  // CTA 0: x, r, z, p and M^-1 (when it fits) of the sub-block
+  extern __shared__ __align__(16) float vec[];  // CTA 0: x, r, z, p and M^-1 of the sub-block
   __shared__ int ctl[2];  // CTA 0's decision: go on; the exponent of the next product
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
@@ -1035,8 +1035,8 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_pcg_solve(PcgSolve v) {
     if constexpr (RES) return slot_sum1<10>(slots, np, e);  // at most 64 tiles: 10 rows
     else return __ldcg(v.qd + o + e);
   };
-  const float *minv = v.Minv32 + CD * CD * (size_t)g0;
-  if (vector_part && v.minv_in_smem) minv = cg_load_minv<CD>(n, minv, vec);
+  const float *minv = nullptr;
+  if (vector_part) minv = cg_load_minv<CD>(n, v.Minv32 + CD * CD * (size_t)g0, vec);
   float mine[RES ? PT : 1];  // this warp's tile, its lane's column
   int ab = 0;
   if constexpr (RES) {
@@ -1781,16 +1781,19 @@ static PcgSolveKernel pcg_solve_kernel(const Ctx *ctx) {
 // The shape of k_pcg_solve: CTAs per cluster C up to eight (the portable size)
 // while all clusters fit the chip at once (one CTA per SM, 152). The register
 // form, eight warps per CTA, when that gives one warp per tile of the largest
-// sub-block (up to 64 tiles, 320 unknowns); else 32 warps per CTA. M^-1 (cd
-// floats per unknown, else an L2 round trip of every step) goes to shared
-// memory beside the vectors while both fit 48 KB.
+// sub-block (up to 64 tiles, 320 unknowns); else 32 warps per CTA. Shared memory
+// holds the vectors and M^-1 (4 + cd floats per unknown; from memory M^-1 was an
+// L2 round trip of every step). Eight CTAs of PCG_FUSED_TILES tiles are at most 31
+// tile rows, and with their 992 unknowns it fits the 48 KB that a launch may use
+// without an attribute, the kernel's static shared memory (below 0.5 KB) included.
+static_assert(PCG_FUSED_TILES * 8 < 32 * 33 / 2, "31 tile rows");
+static_assert(31 * PT * (4 + 8) * sizeof(float) + 1024 <= 48 * 1024, "vectors, M^-1 and static shared memory");
 rpba_status pcg_solve_setup(Ctx *ctx, int max_n) {
   const int n4 = (std::max(max_n, 1) + 3) & ~3;
   const long long tiles = (long long)ctx->max_tiles * (ctx->max_tiles + 1) / 2;
   const size_t vec = (size_t)n4 * 4 * sizeof(float), minv = (size_t)n4 * ctx->cd * sizeof(float);
   ctx->pcg_ff_smem = vec / 2;
-  ctx->pcg_minv_smem = vec + minv <= 48 * 1024 ? 1 : 0;
-  ctx->pcg_solve_smem = vec + (ctx->pcg_minv_smem ? minv : 0);
+  ctx->pcg_solve_smem = vec + minv;
   auto cluster = [&](int warps) {
     int C = 8;
     while (C > 1 && ((long long)(C - 1) * warps >= tiles || (long long)C * ctx->L > 152)) C--;
@@ -1809,7 +1812,7 @@ static rpba_status pcg_solve(Ctx *ctx, int *iters) {
   int *cnt = ctx->counters + PCG_LOOP_COUNTERS;
   const size_t cnt_bytes = (RPBA_PCG_MAX_STAGES + 1) * sizeof(int);
   RPBA_CUDA(cudaMemsetAsync(cnt, 0, cnt_bytes, st));
-  PcgSolve v{ctx->opt.pcg_max_iter, RPBA_PCG_MAX_STAGES, ctx->pcg_minv_smem, ctx->sub_cam_ptr, ctx->ycam_off,
+  PcgSolve v{ctx->opt.pcg_max_iter, RPBA_PCG_MAX_STAGES, ctx->sub_cam_ptr, ctx->ycam_off,
              ctx->npad, ctx->pcg_tiles, ctx->S_off, ctx->pcg_tile_map, ctx->pcg_Shi, ctx->pcg_Slo, ctx->pcg_Minv32,
              ctx->y, ctx->pcg_part, ctx->pcg_q, ctx->pcg_fx, ctx->pcg_x32, ctx->pcg_r32, ctx->pcg_z32, ctx->pcg_p32,
              ctx->pcg_qi, ctx->pcg_st, ctx->pcg_s32, ctx->pcg_act, ctx->pcg_live, cnt, ctx->opt.pcg_tol, RPBA_PCG_INNER_TOL};

@@ -327,11 +327,10 @@ struct Ctx {
   int2 *pcg_tile_map = nullptr;           // per lower tile of the running RCS: (sub-block, a << 16 | b)
   float *pcg_Minv32 = nullptr, *pcg_s32 = nullptr;
   int *pcg_act = nullptr;
-  // the loop as one kernel, k_pcg_solve: whether it is used; CTAs per cluster,
-  // whether M^-1 is in shared memory, whether the tiles stay in registers, its
-  // shared memory
+  // the loop as one kernel, k_pcg_solve: whether it is used, whether the tiles
+  // stay in registers, CTAs per cluster, its shared memory
   bool pcg_fused = false, pcg_res = false;
-  int pcg_cluster = 1, pcg_minv_smem = 0;
+  int pcg_cluster = 1;
   size_t pcg_ff_smem = 0;  // the step kernel's shared memory: r and z of the largest sub-block
   size_t pcg_solve_smem = 0;
   int pcg_pred = 8;        // CG iterations of the previous solve: the first convergence read
