@@ -1201,8 +1201,8 @@ extern "C" rpba_status rpba_covariance(rpba_ctx *h, const int32_t *ids, int32_t 
   const int rows = (int)std::min<size_t>(n, ctx->perm_scratch_n * sizeof(double) / COV_ROW_BYTES);
   double *dout = ctx->perm_scratch;
   int *di = reinterpret_cast<int *>(dout + 9 * (size_t)rows);
-  for (int e0 = 0; e0 < n; e0 += rows) {
-    int m = std::min(rows, n - e0);
+  for (int e0 = 0, m; e0 < n; e0 += m) {
+    m = std::min(rows, n - e0);
     RPBA_CUDA(cudaMemcpyAsync(di, idi.data() + e0, m * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
     RPBA_KERNEL(ctx, "k_covariance", k_covariance<<<nblk(m, 128), 128, 0, ctx->stream>>>(m, di, ctx->R, ctx->t, ctx->intr, ctx->cd == 8 ? ctx->k1 : nullptr, ctx->X,
                                                        ctx->active, ctx->pt_inst_ptr, ctx->pt_inst, ctx->inst_obs_ptr,
