@@ -192,9 +192,10 @@ rpba_status rpba_iterate(rpba_ctx *ctx, int32_t max_outer, rpba_report *report);
 
 /* Autotuner: times candidate launch shapes on the context's own data with
  * CUDA events (5 runs each after one untimed run) and keeps the fastest: the
- * CTA sizes of the intersection (64/128/256 points), the linearisation and the
- * back-substitution (64/128/256 instances) and the robust weights (128/256/512
- * observations), and, for the direct solver, the tensor-core factorisation's
+ * CTA sizes of the intersection (64/128/256 points) and the linearisation
+ * (64/128/256 instances), both in the FP32 form only (the FP64 form's have one
+ * shape), of the back-substitution (64/128/256 instances) and the robust weights
+ * (128/256/512 observations), and, for the direct solver, the tensor-core factorisation's
  * launch form (chol_tc 1 or 2). These kernels give every thread one
  * independent item, so the choice changes timing, not results. The state is
  * unchanged (the intersection's timing restores it). With cache_path (or the

@@ -1737,8 +1737,10 @@ extern "C" rpba_status rpba_tune(rpba_ctx *h, const char *cache_path, int32_t *c
   // the RCS assembly (linearisation), then the back-substitution with trial:
   // per-LM-step scratch only, the state is unchanged
   RPBA_TRY(launch_lm_init(ctx));
-  RPBA_TRY(pick(ctx, &ctx->tune.lin, {64, 128, 256},
-                [&] { return launch_build_rcs(ctx, ctx->lm_lambda, ctx->lm_run); }));
+  // (the FP64 form's linearisation and intersection have one launch shape each)
+  const bool shapes = ctx->opt.precision == 1;
+  auto build_rcs = [&] { return launch_build_rcs(ctx, ctx->lm_lambda, ctx->lm_run); };
+  RPBA_TRY(shapes ? pick(ctx, &ctx->tune.lin, {64, 128, 256}, build_rcs) : build_rcs());
   RPBA_TRY(launch_solve_rcs(ctx, ctx->lm_run, ctx->lm_cholfail));
   RPBA_TRY(pick(ctx, &ctx->tune.backsub, {64, 128, 256}, [&] { return launch_backsub_trial(ctx, ctx->lm_run); }));
   // the direct solve's factorisation: persistent or one launch per step
@@ -1750,7 +1752,7 @@ extern "C" rpba_status rpba_tune(rpba_ctx *h, const char *cache_path, int32_t *c
     RPBA_TRY(st);
   }
   // the TP intersection from the saved state every time
-  {
+  if (shapes) {
     rpba_status st = pick(ctx, &ctx->tune.isect, {64, 128, 256}, [&]() -> rpba_status {
       RPBA_TRY(restore());
       return launch_intersect(ctx, 1, nullptr);
