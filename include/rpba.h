@@ -205,6 +205,14 @@ rpba_status rpba_iterate(rpba_ctx *ctx, int32_t max_outer, rpba_report *report);
  * unwritable cache, CUDA. */
 rpba_status rpba_tune(rpba_ctx *ctx, const char *cache_path, int32_t *chosen);
 
+/* How long a thread block of the direct solvers' kernels waits for what another
+ * one (or another warp) writes before it gives up: limit_ns nanoseconds (default
+ * 500 ms) and 64 polls; 0: the substitution looks once. (chol_tc 1 and 2 keep
+ * 200 ms in their factorisation.) A wait that runs out ends the call (rpba_bact,
+ * rpba_iterate, rpba_lm_step, ...) with DEVICE_TIMEOUT, its LM step rejected. Not a
+ * step of the paper's method. Errors: INVALID_ARG for a negative limit. */
+rpba_status rpba_set_wait_limit(rpba_ctx *ctx, int64_t limit_ns);
+
 /* One outer iteration of the RPBA loop (Sec. 5) in steady state: the LM
  * adjustment of every sub-block (Eq. bact, up to options.max_inner lock-step
  * LM iterations), the exchange of cameras and single-sub-block points, the

@@ -47,6 +47,8 @@ struct CholView {
   int *fail;
   const int *sched;      // per step k: L+1 prefix sums of panel tiles, of update tiles and of 2 x 2 blocks of them
   int L;
+  int *late;             // set when a bounded wait ran out (the host reports it)
+  uint64_t wait_ns;      // its limit
 };
 
 // p -> (a, b), b <= a, p = a (a + 1) / 2 + b; FP32 estimate, exact integer fix-up
@@ -128,7 +130,8 @@ __device__ __forceinline__ double rcp_ulp(double x) {
 // ---------------------------------------------------------------------------
 // The inverse Cholesky factor of a 32 x 32 SPD tile (smem C, CLD stride, both
 // triangles of the part used: the lower one), by the whole CTA (256 threads),
-// into out (row-major, CT stride). False (uniform) on a non-positive pivot.
+// into out (row-major, CT stride). False (uniform) on a non-positive pivot, and
+// when a wait ran out (cv.late).
 // Elimination of [C | I] gives L^-1 beside the factor. The factorisation's next
 // step waits for this tile.
 //
@@ -160,7 +163,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
 }
 
-__device__ bool cta_inverse_factor(const double *C, double *out) {
+__device__ bool cta_inverse_factor(const double *C, double *out, const CholView &cv) {
   __shared__ double Ls[CT][CT], dv[CT];
   __shared__ __align__(8) uint64_t ready[CT];  // column j of Ls and dv[j] are there
   __shared__ int late;
@@ -189,7 +192,7 @@ __device__ bool cta_inverse_factor(const double *C, double *out) {
 #pragma unroll 1
     for (int jw = 0; jw < 8; jw++) {
       const int j = 8 * jb + jw;
-      if (in_time) in_time = tc::mbar_wait(&ready[j], 0, 500000000ull);
+      if (in_time) in_time = tc::mbar_wait(&ready[j], 0, cv.wait_ns);
       const double l = lane > j ? Ls[j][lane] : 0.0;
       // column j + 1 first, by its owner
       const bool own = j + 1 < CT && w == ((j + 1) & 7);
@@ -217,6 +220,7 @@ __device__ bool cta_inverse_factor(const double *C, double *out) {
   __syncthreads();
   const double d = dv[lane];
   const bool ok = __all_sync(0xffffffffu, d > 0.0);
+  if (late && threadIdx.x == 0) atomicExch(cv.late, 1);
   if (!ok || late) return false;
   const double rs = rsqrt(d);
 #pragma unroll
@@ -234,7 +238,7 @@ __device__ __forceinline__ float div_by(float a, float d, float r) {
   return fmaf(fmaf(-q, d, a), r, q);
 }
 
-__device__ bool cta_inverse_factor(const float *C, float *out) {
+__device__ bool cta_inverse_factor(const float *C, float *out, const CholView &) {
   __shared__ float Ls[CT][CT];  // column j of L
   __shared__ float dg[CT], rdg[CT];
   __shared__ int bad;
@@ -305,7 +309,7 @@ __global__ void __launch_bounds__(256) k_chol_first(T *S, T *Linv, CholView cv) 
   __shared__ T C[CT * CLD];
   for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) C[(e / CT) * CLD + e % CT] = A[(size_t)(e / CT) * np + e % CT];
   __syncthreads();
-  if (!cta_inverse_factor(C, Linv + cv.linv_off[l]) && threadIdx.x == 0) cv.fail[l] = 1;
+  if (!cta_inverse_factor(C, Linv + cv.linv_off[l], cv) && threadIdx.x == 0) cv.fail[l] = 1;
 }
 
 // 32 x 32 x 32 product on 256 threads, 2 x 2 outputs per thread:
@@ -422,7 +426,7 @@ __global__ void __launch_bounds__(256, 4) k_chol_update(T *S, T *Linv, CholView 
         P[rr * CLD + cc] = A[(size_t)((k + 1) * CT + rr) * np + (k + 1) * CT + cc] - acc[r][c];
       }
     __syncthreads();
-    if (!cta_inverse_factor(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT) && threadIdx.x == 0)
+    if (!cta_inverse_factor(P, Linv + cv.linv_off[l] + (size_t)(k + 1) * CT * CT, cv) && threadIdx.x == 0)
       cv.fail[l] = 1;
     return;
   }
@@ -827,8 +831,8 @@ __global__ void __launch_bounds__(128) k_chol_tc_persistent(const __grid_constan
 // m >= k + TR - TS and is done with x_k if TR >= TS + 2.
 #define TS 8
 #define TR 16          // slots of the ring
+#define TRSV_DRAIN_NS 100000ull  // a store between SMs takes about a microsecond
 #define TRSV_PRE 4     // owned tiles of the next step in registers (more are read late)
-#define TRSV_WAIT_NS 500000000ull
 static_assert(TR >= TS + 2, "a slot is free when it is written again");
 
 // thread part of eight: (4 c .. 4 c + 3) . v
@@ -856,11 +860,21 @@ __device__ inline uint32_t map_rank(uint32_t addr, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// phase of a barrier that other CTAs of the cluster complete
+// phase of a barrier that other CTAs of the cluster complete (limit 0: one look; a
+// try may suspend the thread until the phase is over)
 __device__ inline bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
-  uint64_t t0 = 0;
-  for (;;) {
-    uint32_t ok;
+  uint32_t ok;
+  if (limit_ns == 0) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(tc::smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+  }
+  return tc::bounded_wait(limit_ns, [&] {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
@@ -868,11 +882,8 @@ __device__ inline bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, uint64_
         : "=r"(ok)
         : "r"(tc::smem_u32(bar)), "r"(parity)
         : "memory");
-    if (ok) return true;
-    uint64_t t = tc::global_ns();
-    if (t0 == 0) t0 = t;
-    if (t - t0 > limit_ns) return false;
-  }
+    return ok != 0;
+  });
 }
 
 static size_t trsv_smem(int tiles, size_t elem) { return (size_t)((tiles + TS - 1) / TS) * CT * elem; }
@@ -914,7 +925,7 @@ __global__ void __cluster_dims__(TS, 1, 1) __launch_bounds__(256)
   // entries of the step (this thread's four), in place for all CTAs
   auto receive = [&](int dir, int step, T *xv) {
     int s = step % TR;
-    if (ok) ok = mbar_wait_cluster(&bar[dir][s], (step / TR) & 1, TRSV_WAIT_NS);
+    if (ok) ok = mbar_wait_cluster(&bar[dir][s], (step / TR) & 1, cv.wait_ns);
 #pragma unroll
     for (int c = 0; c < 4; c++) xv[c] = ring[dir][s][part * 4 + c];
     if (tid == 0 && ok && step + TR < nt) tc::mbar_arrive_expect_tx(&bar[dir][s], CT * sizeof(T));
@@ -1046,8 +1057,13 @@ __global__ void __cluster_dims__(TS, 1, 1) __launch_bounds__(256)
 #pragma unroll
       for (int c = 0; c < 4; c++) pre[m][c] = nxt[m][c];
   }
-  if (!ok) cv.fail[l] = 1;
-  cluster.sync();  // stores into this CTA's ring are in before it leaves
+  if (!ok) {
+    cv.fail[l] = 1;
+    atomicExch(cv.late, 1);
+  }
+  const bool drain = __syncthreads_or(!ok);
+  cluster.sync();  // every store into this CTA's ring is issued, and in if no wait ran out
+  if (drain) tc::bounded_wait(TRSV_DRAIN_NS, [] { return false; });  // else given time to land before the CTA leaves
 }
 
 template <typename T>
@@ -1215,8 +1231,6 @@ rpba_status tc_chol_setup(Ctx *ctx) {
   RPBA_TRY(ctx_alloc(ctx, (void **)&ctx->tc_sched, sizeof(int) * sched.size()));
   RPBA_CUDA(cudaMemcpyAsync(ctx->tc_sched, sched.data(), sizeof(int) * sched.size(), cudaMemcpyHostToDevice,
                             ctx->stream));
-  RPBA_TRY(ctx_alloc(ctx, (void **)&ctx->tc_err, sizeof(int)));
-  RPBA_CUDA(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->stream));
   // cuTensorMapEncodeTiled through the runtime (no link against the driver library)
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult q;
@@ -1283,7 +1297,7 @@ rpba_status tc_chol_setup(Ctx *ctx) {
 // the FP32 factorisation of every running sub-block on the tensor cores
 static rpba_status factor_tc(Ctx *ctx, float *S, float *Linv, const long long *off, const int *run, int *fail) {
   TcView tv{S, off, ctx->npad, Linv, ctx->linv_off, run, fail, ctx->tc_panel[0], ctx->tc_panel[1],
-            ctx->tc_panel[2], ctx->tc_prow, nullptr, ctx->L, ctx->tc_err,
+            ctx->tc_panel[2], ctx->tc_prow, nullptr, ctx->L, ctx->counters + WAIT_LATE,
             ctx->tc_tasks, ctx->tc_n_tasks, ctx->tc_count, ctx->tc_count + 1, ctx->tc_need, ctx->max_tiles};
   if (ctx->opt.chol_tc == 2) {  // one persistent cooperative launch
     RPBA_CUDA(cudaMemsetAsync(ctx->tc_count, 0, sizeof(int) * (1 + (size_t)ctx->L * ctx->max_tiles), ctx->stream));
@@ -1320,7 +1334,8 @@ rpba_status launch_solve_rcs(Ctx *ctx, const int *run_dev, int *fail_dev) {
   if (T_max == 0) return RPBA_OK;
   if (ctx->opt.solver != 2) {
     // FP64 direct: factor S in place, one forward/backward solve
-    CholView cv{ctx->S_off, ctx->npad, ctx->linv_off, run_dev, fail_dev, ctx->sched, ctx->L};
+    CholView cv{ctx->S_off,  ctx->npad, ctx->linv_off, run_dev, fail_dev, ctx->sched, ctx->L, ctx->counters + WAIT_LATE,
+                ctx->wait_ns};
     RPBA_TRY(factor<double>(ctx, ctx->S, ctx->Linv64, cv, T_max));
     RPBA_CUDA(cudaMemcpyAsync(ctx->dC, ctx->y, ctx->ytot * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     RPBA_TRY(trsv<double>(ctx, "k_trsv_f64", ctx->S, ctx->Linv64, cv, ctx->dC));
@@ -1335,7 +1350,8 @@ rpba_status launch_solve_rcs(Ctx *ctx, const int *run_dev, int *fail_dev) {
               k_mixed_convert<<<dim3(64, ctx->L), 256, 0, ctx->stream>>>(ctx->S, ctx->S32, ctx->S_off, ctx->S32_off,
                                                                          ctx->npad, ctx->ycam_off, run_dev,
                                                                          ctx->ir_d));
-  CholView cv{ctx->S32_off, ctx->npad, ctx->linv_off, run_dev, fail_dev, ctx->sched, ctx->L};
+  CholView cv{ctx->S32_off, ctx->npad, ctx->linv_off, run_dev, fail_dev, ctx->sched, ctx->L, ctx->counters + WAIT_LATE,
+              ctx->wait_ns};
   if (ctx->opt.chol_tc && ctx->tc_ready)
     RPBA_TRY(factor_tc(ctx, ctx->S32, ctx->Linv32, ctx->S32_off, run_dev, fail_dev));
   else

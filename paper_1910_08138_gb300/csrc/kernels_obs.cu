@@ -2446,7 +2446,7 @@ rpba_status launch_lm_decide(Ctx *ctx) {
   RPBA_KERNEL(ctx, "k_lm_decide", k_lm_decide<<<nblk(ctx->L, 128), 128, 0, ctx->stream>>>(
       ctx->L, ctx->opt.lambda0, ctx->opt.stop_ratio, ctx->opt.max_inner, ctx->opt.max_reject, ctx->lm_lambda,
       ctx->lm_F, ctx->lm_Ft, ctx->lm_best, ctx->lm_grace, ctx->lm_rej, ctx->lm_it, ctx->lm_run, ctx->lm_acc,
-      ctx->lm_cholfail, ctx->counters));
+      ctx->lm_cholfail, ctx->counters + LM_RUNNING));
   return RPBA_OK;
 }
 

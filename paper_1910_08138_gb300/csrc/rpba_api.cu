@@ -792,7 +792,9 @@ static rpba_status build(Ctx *ctx, const rpba_problem *pb) {
   }
   RPBA_TRY(alloc_n(ctx, &ctx->red, (size_t)ctx->red_blocks * 6 + 16));
   RPBA_TRY(alloc_n(ctx, &ctx->counters, 32));
+  RPBA_CUDA(cudaMemsetAsync(ctx->counters, 0, 32 * sizeof(int), ctx->stream));
   RPBA_CUDA(cudaMallocHost((void **)&ctx->h_pinned_counter, 32 * sizeof(int)));
+  memset(ctx->h_pinned_counter, 0, 32 * sizeof(int));
   RPBA_CUDA(cudaMallocHost((void **)&ctx->h_pinned_d, 16 * sizeof(double)));
   // state: rotations from the poses, unit weights, instance copies at X
   if (M) RPBA_KERNEL(ctx, "k_pose_to_R", k_pose_to_R<<<nblk(M, 128), 128, 0, ctx->stream>>>(M, pose_d, ctx->R, ctx->t));
@@ -1247,6 +1249,24 @@ extern "C" rpba_status rpba_rcs(rpba_ctx *h, int32_t l, double lambda, double *S
   return RPBA_OK;
 }
 
+// after the stream has been synchronised: an error when a wait of the solve ran
+// out (its sub-blocks count as failed; the LM step rejects them)
+static rpba_status wait_check(Ctx *ctx) {
+  if (!ctx->h_pinned_counter[WAIT_LATE]) return RPBA_OK;
+  RPBA_CUDA(cudaMemsetAsync(ctx->counters + WAIT_LATE, 0, sizeof(int), ctx->stream));
+  RPBA_TRY(sync(ctx));
+  ctx->h_pinned_counter[WAIT_LATE] = 0;
+  ctx->err = "a wait inside the factorisation or the substitution of the reduced camera system ran out";
+  return RPBA_ERR_DEVICE_TIMEOUT;
+}
+
+static rpba_status wait_read(Ctx *ctx) {
+  RPBA_CUDA(cudaMemcpyAsync(ctx->h_pinned_counter + WAIT_LATE, ctx->counters + WAIT_LATE, sizeof(int),
+                            cudaMemcpyDeviceToHost, ctx->stream));
+  RPBA_TRY(sync(ctx));
+  return wait_check(ctx);
+}
+
 // one lock-step LM iteration of the running sub-blocks
 static rpba_status lm_iteration(Ctx *ctx) {
   RPBA_TRY(launch_build_rcs(ctx, ctx->lm_lambda, ctx->lm_run));
@@ -1278,7 +1298,7 @@ extern "C" rpba_status rpba_lm_step(rpba_ctx *h, double lambda, int32_t *accepte
   std::vector<double> dCh(ytot);
   if (dc && ytot)
     RPBA_CUDA(cudaMemcpyAsync(dCh.data(), ctx->dC, ytot * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-  RPBA_TRY(sync(ctx));
+  RPBA_TRY(wait_read(ctx));
   std::vector<int> acc(L);
   for (int l = 0; l < L; l++) {
     if (!run[l]) acc[l] = 0;
@@ -1316,10 +1336,12 @@ extern "C" rpba_status rpba_lm_step(rpba_ctx *h, double lambda, int32_t *accepte
 // and the running count for the host
 static rpba_status lm_post(Ctx *ctx) {
   RPBA_TRY(launch_backsub_trial(ctx, ctx->lm_run));
-  RPBA_CUDA(cudaMemsetAsync(ctx->counters, 0, sizeof(int), ctx->stream));
+  RPBA_CUDA(cudaMemsetAsync(ctx->counters + LM_RUNNING, 0, sizeof(int), ctx->stream));
   RPBA_TRY(launch_lm_decide(ctx));
   RPBA_TRY(launch_lm_apply(ctx, ctx->lm_acc));
-  RPBA_CUDA(cudaMemcpyAsync(ctx->h_pinned_counter, ctx->counters, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  static_assert(WAIT_LATE == LM_RUNNING + 1, "one copy");
+  RPBA_CUDA(cudaMemcpyAsync(ctx->h_pinned_counter + LM_RUNNING, ctx->counters + LM_RUNNING, 2 * sizeof(int),
+                            cudaMemcpyDeviceToHost, ctx->stream));
   return RPBA_OK;
 }
 
@@ -1556,7 +1578,8 @@ static rpba_status run_bact(Ctx *ctx, int *inner_total, int *launches) {
   for (;;) {
     RPBA_TRY(lm_step_run(ctx));
     n++;
-    if (ctx->h_pinned_counter[0] == 0) break;
+    RPBA_TRY(wait_check(ctx));
+    if (ctx->h_pinned_counter[LM_RUNNING] == 0) break;
     if (n > 100000) { ctx->err = "LM loop did not terminate"; return RPBA_ERR_NOT_CONVERGED; }
   }
   std::vector<int> it(ctx->L);
@@ -1768,7 +1791,7 @@ extern "C" rpba_status rpba_tune(rpba_ctx *h, const char *cache_path, int32_t *c
       free_graph(g);
       g = nullptr;
     }
-  RPBA_TRY(sync(ctx));
+  RPBA_TRY(wait_read(ctx));
   if (chosen) {
     chosen[0] = ctx->tune.isect;
     chosen[1] = ctx->tune.lin;
@@ -1778,6 +1801,14 @@ extern "C" rpba_status rpba_tune(rpba_ctx *h, const char *cache_path, int32_t *c
   }
   const char *path = cache_path ? cache_path : ctx->opt.tune_cache;
   if (path && *path) RPBA_TRY(tune_store(ctx, path));
+  return RPBA_OK;
+}
+
+extern "C" rpba_status rpba_set_wait_limit(rpba_ctx *h, int64_t limit_ns) {
+  CTX_OR_FAIL;
+  if (limit_ns < 0) return RPBA_ERR_INVALID_ARG;
+  ctx->wait_ns = (uint64_t)limit_ns;
+  free_lm_graphs(ctx);  // captured graphs carry the old limit
   return RPBA_OK;
 }
 

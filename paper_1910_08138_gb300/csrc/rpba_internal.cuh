@@ -389,13 +389,12 @@ struct Ctx {
   // columns of 32 as three TF32 pieces in panel-major order (block column k
   // of sub-block l is npad_l rows of 32 floats from row tc_prow[l] + k npad_l),
   // a TMA tensor map per piece, per step the CTA prefix sums over the
-  // sub-blocks, and a flag that a bounded wait gave up
+  // sub-blocks
   float *tc_panel[3] = {nullptr, nullptr, nullptr};
   long long *tc_prow = nullptr;
   int *tc_sched = nullptr;
   std::vector<int> h_tc_ctas;  // CTAs of each step
   CUtensorMap tc_map[3];
-  int *tc_err = nullptr;
   bool tc_ready = false;
   // persistent form: the task queue, tasks per (sub-block, step), the queue
   // head and finished-task counters, the grid (resident CTAs)
@@ -417,6 +416,7 @@ struct Ctx {
   double *red = nullptr;   // scratch for block partials
   int red_blocks = 0;
   int *counters = nullptr; // small device counters
+  uint64_t wait_ns = 500000000;  // limit of a kernel's wait for another thread block or warp
   // profiling: kernel launch counts (always) and event-timed phases (when enabled)
   long long launches = 0;
   std::map<std::string, long long> launch_by_name;
@@ -585,6 +585,10 @@ rpba_status launch_robust_weights(Ctx *ctx, int *n_down);
 rpba_status launch_eliminate(Ctx *ctx);
 rpba_status launch_sub_costs(Ctx *ctx, int trial, double *F_dev);
 rpba_status launch_build_rcs(Ctx *ctx, const double *lambda_dev, const int *run_dev);
+// device counters read after every LM step: the sub-blocks still running, and
+// whether a bounded wait of the solve ran out
+#define LM_RUNNING 4
+#define WAIT_LATE 5
 rpba_status launch_solve_rcs(Ctx *ctx, const int *run_dev, int *fail_dev);
 rpba_status tc_chol_setup(Ctx *ctx);
 rpba_status launch_pcg_blockjacobi(Ctx *ctx, const int *run_dev, int *fail_dev);

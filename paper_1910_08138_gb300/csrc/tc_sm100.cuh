@@ -52,14 +52,22 @@ __device__ inline bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   return ok != 0;
 }
 
-// waits for the phase with the given parity to complete; false after
-// `limit_ns` nanoseconds without completion
+// polls until done() or, false, until MBAR_POLLS polls and `limit_ns` nanoseconds
+// are over: time alone also passes while the GPU runs another process
+#define MBAR_POLLS 64
+template <class F>
+__device__ inline bool bounded_wait(uint64_t limit_ns, F done) {
+  if (done()) return true;
+  const uint64_t t0 = global_ns();
+  for (uint32_t n = 1;; n++) {
+    if (n >= MBAR_POLLS && global_ns() - t0 >= limit_ns) return false;
+    if (done()) return true;
+  }
+}
+
+// waits for the phase with the given parity to complete
 __device__ inline bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  uint64_t t0 = global_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (global_ns() - t0 > limit_ns) return false;
-  return true;
+  return bounded_wait(limit_ns, [&] { return mbar_try_wait(bar, parity); });
 }
 
 // ---------------------------------------------------------------------------

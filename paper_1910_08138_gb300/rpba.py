@@ -116,6 +116,7 @@ def load(build_if_missing: bool = True):
         "rpba_profile_enable": (C.c_int, [vp, C.c_int32]),
         "rpba_profile_select": (C.c_int, [vp, C.c_char_p]),
         "rpba_tune": (C.c_int, [vp, C.c_char_p, _ip]),
+        "rpba_set_wait_limit": (C.c_int, [vp, C.c_int64]),
         "rpba_partition": (C.c_int, [C.c_int32, C.c_int32, C.c_int32, _ip, _ip, C.c_int32, _ip, _dp,
                                      C.POINTER(C.c_double)]),
         "rpba_get_camera_rt": (C.c_int, [vp, _dp, _dp]),
@@ -466,6 +467,11 @@ class Rpba:
         dc, dx = np.zeros(self.cd * self.M), np.zeros((self.P, 3))
         self._c(load().rpba_lm_step(self._h, float(lam), _i(acc), _d(Fb), _d(Ft), _d(dc), _d(dx)))
         return acc, Fb, Ft, dc, dx
+
+    def set_wait_limit(self, limit_ns):
+        """Longest wait of a thread block for another one in the direct solvers'
+        kernels, in nanoseconds (0: the substitution looks once); RpbaError when one runs out."""
+        self._c(load().rpba_set_wait_limit(self._h, int(limit_ns)))
 
     def tune(self, cache_path=None):
         """Autotune the launch shapes on this context's data; returns the
