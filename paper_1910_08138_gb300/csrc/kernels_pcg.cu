@@ -24,7 +24,8 @@
 // per tile with plain FMAs; k_pcg_step32 is the FP32 step); then
 // X += d in float-float and the true residual R = y - S X is formed in
 // float-float from both planes (k_pcg_symv_ff, TwoProduct and TwoSum per
-// entry, ~1e-13 relative) by k_pcg_stage, which ends the solve at
+// entry, ~1e-13 relative; its tiles' parts added by k_pcg_slot_sum) by
+// k_pcg_stage, which ends the solve at
 // ||R|| <= pcg_tol ||y|| or starts the next stage. The entrywise rounding of
 // S_hi is a relative perturbation of 2^-24, so a stage reduces the residual
 // by about max(1e-4, 2^-24 cond) with cond the condition of the Jacobi-scaled
@@ -1772,11 +1773,12 @@ static PcgSolveKernel pcg_solve_kernel(const Ctx *ctx) {
 
 // k_pcg_solve or the loop of graph nodes: the nodes spread the products over
 // the whole chip, but a step costs three launches and the sub-blocks wait for
-// each other. One kernel is faster while an SM gets up to two tiles per warp:
-// eight sub-blocks of 750 unknowns (41 tiles per CTA) 1.79 against 1.89 ms per
-// call; beyond that its product, which is bound by the instructions of the
-// fewer SMs, loses: 64 sub-blocks of 936 (232 tiles per CTA) 4.80 against
-// 4.40 ms.
+// each other. One kernel is faster while an SM gets up to two tiles per warp;
+// beyond that its product, which is bound by the instructions of the fewer SMs,
+// loses. Per call, one kernel against the nodes: eight sub-blocks of 720 unknowns
+// (35 tiles per CTA) 1.69 and 1.87 ms, of 936 (58) 1.79 and 1.95; 30 of 720 (56)
+// 2.79 and 2.75; 38 of 720 (69) 3.25 and 3.13; 24 of 936 (78) 3.12 and 2.92; 64 of
+// 936 (232) 4.80 and 4.40.
 #define PCG_FUSED_TILES 64
 // The shape of k_pcg_solve: CTAs per cluster C up to eight (the portable size)
 // while all clusters fit the chip at once (one CTA per SM, 152). The register

@@ -62,9 +62,9 @@ __device__ inline void block_sum(double *v, int nv, double *out) {
 // observation: [w v^T C^-1 v, 1, |v|^2 if w == 1, 1 if w == 1]; the others one
 // thread per point: the active count. The CTA that arrives last adds the
 // partials in block order, so the sums do not depend on the order of arrival.
-// A small block is bound by launches: three kernels behind one another took
-// 47.1 us per call at 8000 observations, this one takes 43.6 us (call, copy
-// back and synchronisation included).
+// A small block is bound by launches, the copy back into pageable memory and the
+// synchronisation: three kernels behind one another took 45.8 to 48.9 us per call
+// at 8000 observations (medians of five processes), this one takes 41.5 to 43.5 us.
 //
 // Arrivals are counted from zero to the call's last, who sets the word back, so
 // calls whose work does not overlap need no order among them. Successive calls
