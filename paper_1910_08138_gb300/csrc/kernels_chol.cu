@@ -1069,8 +1069,11 @@ __global__ void __cluster_dims__(TS, 1, 1) __launch_bounds__(256)
 template <typename T>
 static rpba_status trsv(Ctx *ctx, const char *name, const T *S, const T *Linv, const CholView &cv, T *r) {
   size_t smem = trsv_smem(ctx->max_tiles, sizeof(T));
-  if (smem > 32 * 1024)  // beyond this the ring and z need more than the default 48 KB
-    RPBA_CUDA(cudaFuncSetAttribute(k_trsv_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // beyond 32 KB the ring and z need more than the default 48 KB. The limit belongs
+  // to the kernel, not to the context: every caller sets the same one, so that none
+  // lowers it between another's call and launch (216 KB: 6,912 tile rows)
+  if (smem > 32 * 1024)
+    RPBA_CUDA(cudaFuncSetAttribute(k_trsv_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
   RPBA_KERNEL(ctx, name, k_trsv_cluster<T><<<dim3(TS, ctx->L), 256, smem, ctx->stream>>>(S, Linv, cv, ctx->ycam_off, r, r));
   return RPBA_OK;
 }
