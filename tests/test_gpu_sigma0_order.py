@@ -34,7 +34,7 @@ def test_a_call_that_waits_on_its_stream_gets_its_own_sums(sizes):
         got = [None, None]
         torch.cuda.synchronize()
         with torch.cuda.stream(waiting):
-            torch.cuda._sleep(400_000_000)  # about 0.2 s: the call below is entered, its work waits
+            torch.cuda._sleep(1_000_000_000)  # about 0.5 s: the call below is entered, its work waits
 
         def call():
             got[0] = rpba.rpba_sigma0_noalloc(*early, stream=waiting)[2]
